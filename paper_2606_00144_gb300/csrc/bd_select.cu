@@ -21,15 +21,15 @@
 //               max score finds the bin holding the k-th largest; that bin's few items are
 //               ranked exactly by (score desc, position asc) (4-pass radix select on the
 //               fp32 bits when the bin is crowded); then an ascending compaction (warp
-//               ballots + block scan) with sinks and recents.  Four kernels of that
-//               method: topk_rows_kernel (token level, up to 16K middle positions, every
-//               score in registers), topk_rows_chunk_kernel (chunk level, up to 16K chunks,
-//               every chunk score in registers), topk_token_kernel (token level, up to 32K,
-//               scores in shared memory) and topk_kernel (longer middles of either level).
+//               ballots + block scan) with sinks and recents.  topk_rows_kernel (token level)
+//               and topk_rows_chunk_kernel (chunk level) here hold every item of a middle of up
+//               to 16K positions in registers, topk_token_kernel up to 32K in shared memory;
+//               bd_topk_long.cu spreads longer middles over a cluster.
 #include <algorithm>
 
 #include "bd_common.cuh"
 #include "bd_internal.h"
+#include "bd_topk.cuh"
 
 namespace bd {
 
@@ -37,10 +37,6 @@ constexpr int kSKeys = 128;          // keys per tile (UMMA M)
 constexpr int kSThreads = 576;       // producer, MMA, 4 x 4 epilogue warps
 constexpr int kMaxAcc = 4;           // TMEM accumulators (<= 512 columns)
 constexpr int kSQOffset = 12288;     // shared-memory offset of the window-query tiles
-constexpr int kTopkThreads = 1024;
-constexpr int kTopkSmemBytes = 200 * 1024;   // item values staged in shared memory up to this size
-constexpr int kBins = 4096;                   // linear histogram bins of the value range
-constexpr int kBinCandMax = 2048;             // items of the boundary bin ranked exactly
 
 struct ScoreParams {
   const __nv_bfloat16* q_win;   // [units * nq_rows][D]
@@ -727,361 +723,10 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
 
 // ============================================================================ top-B select
 
-struct TopkParams {
-  const float* score;      // [units][n_mid_pad]
-  int32_t* idx_out;        // [units][budget]
-  int32_t* count_out;      // [units]
-  int t_ctx, budget, n_sink, n_recent, chunk, n_mid_pad;
-  int keep_all;            // budget >= t_ctx
-  int smem_items;          // item values staged in shared memory when n_items <= smem_items
-  const int32_t* seq_lens; // per-sequence context lengths [batch] or null (all t_ctx)
-  int h_kv;
-  int* status;
-};
-
-// A unit whose context fits the budget keeps every position (the B >= T rule).
-__device__ __forceinline__ bool topk_keep_all(const TopkParams& p, int unit, int t_u, int32_t* out) {
-  if (!p.keep_all && p.budget < t_u) return false;
-  for (int i = threadIdx.x; i < p.budget; i += blockDim.x) out[i] = i < t_u ? i : -1;
-  if (threadIdx.x == 0) p.count_out[unit] = t_u;
-  return true;
-}
-
-// Exclusive scan of one value per warp (32 warps), result broadcast through smem.
-__device__ __forceinline__ uint32_t warp_totals_exclusive(uint32_t v, uint32_t* wsum, uint32_t* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) wsum[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    const uint32_t w = wsum[lane];
-    uint32_t incl = w;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += y;
-    }
-    wsum[lane] = incl - w;
-    if (lane == 31) *total = incl;
-  }
-  __syncthreads();
-  const uint32_t r = wsum[warp];
-  __syncthreads();
-  return r;
-}
-
-__global__ void __launch_bounds__(kTopkThreads, 1) topk_kernel(const TopkParams p) {
-  extern __shared__ uint32_t vals[];           // item values (fp32 bits) | candidates | samples
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t wsum[32];
-  __shared__ uint32_t s_total, s_prefix, s_krem;
-  grid_dependency_wait();
-  allow_dependent_launch();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int unit = blockIdx.x;
-  int32_t* out = p.idx_out + (size_t)unit * p.budget;
-
-  const int t_u = unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
-  if (topk_keep_all(p, unit, t_u, out)) return;
-  const int lo = p.n_sink, hi = t_u - p.n_recent;
-  const int s = p.chunk;
-  const int free = p.budget - p.n_sink - p.n_recent;
-  const int c_first = lo / s;
-  const int n_items = (hi > lo) ? ((hi - 1) / s - c_first + 1) : 0;
-  const int k = min(free / s, n_items);
-  const float* sc = p.score + (size_t)unit * p.n_mid_pad;
-  const bool take_all = (k >= n_items), take_none = (k <= 0);
-  const bool ranked = !take_all && !take_none;
-  const bool staged = n_items <= p.smem_items;
-
-  auto members = [&](int i, int& a, int& b) {
-    const int c = c_first + i;
-    a = max(c * s, lo);
-    b = min(c * s + s, hi);
-  };
-  // a chunk's score: its members summed in position order, their loads issued eight at a
-  // time (all in flight together; the zeros past b add nothing to a sum of scores >= +0)
-  auto value_global = [&](int i) -> uint32_t {
-    if (s == 1) return __float_as_uint(__ldcg(sc + i));
-    int a, b;
-    members(i, a, b);
-    float v = 0.f;
-    for (int q0 = a; q0 < b; q0 += 8) {
-      float t[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) t[j] = q0 + j < b ? __ldcg(sc + (q0 + j - lo)) : 0.f;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v += t[j];
-    }
-    return __float_as_uint(v);
-  };
-  if (ranked && staged) {
-    if (s == 1) {
-      const int n4 = n_items / 4;
-      const float4* sc4 = reinterpret_cast<const float4*>(sc);
-      for (int i = tid; i < n4; i += kTopkThreads) {
-        const float4 v = __ldcg(sc4 + i);
-        vals[4 * i] = __float_as_uint(v.x);
-        vals[4 * i + 1] = __float_as_uint(v.y);
-        vals[4 * i + 2] = __float_as_uint(v.z);
-        vals[4 * i + 3] = __float_as_uint(v.w);
-      }
-      for (int i = 4 * n4 + tid; i < n_items; i += kTopkThreads) vals[i] = __float_as_uint(__ldcg(sc + i));
-    } else {
-      // two chunks per round, so that both chunks' loads are in flight together
-      for (int i = tid; i < n_items; i += 2 * kTopkThreads) {
-        const int i2 = i + kTopkThreads;
-        const uint32_t v1 = value_global(i);
-        const uint32_t v2 = i2 < n_items ? value_global(i2) : 0u;
-        vals[i] = v1;
-        if (i2 < n_items) vals[i2] = v2;
-      }
-    }
-    __syncthreads();
-  }
-  auto val = [&](int i) -> uint32_t { return staged ? vals[i] : value_global(i); };
-
-  // ---- value bits of the k-th largest item (tau) and how many items equal to tau to take (krem)
-  // Linear histogram between the block's min and max value: bins are monotone in the value,
-  // so the k-th largest lies in the bin where the count from the top reaches k; its items
-  // are few and are ranked exactly by (value desc, position asc).
-  uint32_t prefix = 0, krem = (uint32_t)k;
-  bool found = false, simple_eq = false;
-  if (ranked && staged) {
-    uint32_t* bins = reinterpret_cast<uint32_t*>(vals + ((p.smem_items + 1) & ~1));   // [kBins]
-    uint64_t* cand = reinterpret_cast<uint64_t*>(bins + kBins);                       // [kBinCandMax]
-    float lmin = INFINITY, lmax = -INFINITY;
-    for (int i = tid; i < n_items; i += kTopkThreads) {
-      const float v = __uint_as_float(vals[i]);
-      lmin = fminf(lmin, v);
-      lmax = fmaxf(lmax, v);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      lmin = fminf(lmin, __shfl_xor_sync(0xffffffffu, lmin, off));
-      lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
-    }
-    __shared__ float s_min[32], s_max[32];
-    __shared__ uint32_t s_bin, s_above, s_nc, s_taukey, s_eq_take, s_eq_all;
-    if (lane == 0) {
-      s_min[warp] = lmin;
-      s_max[warp] = lmax;
-    }
-    for (int i = tid; i < kBins; i += kTopkThreads) bins[i] = 0;
-    if (tid == 0) {
-      s_nc = 0;
-      s_eq_take = 0;
-      s_eq_all = 0;
-      s_bin = 0xFFFFFFFFu;
-    }
-    __syncthreads();
-    float vmin = s_min[0], vmax = s_max[0];
-    for (int w = 1; w < 32; ++w) {
-      vmin = fminf(vmin, s_min[w]);
-      vmax = fmaxf(vmax, s_max[w]);
-    }
-    const float scale = vmax > vmin ? (float)(kBins - 1) / (vmax - vmin) : 0.f;
-    auto bin_of = [&](uint32_t u) -> int {
-      return min(kBins - 1, (int)((__uint_as_float(u) - vmin) * scale));
-    };
-    for (int i = tid; i < n_items; i += kTopkThreads) atomicAdd(&bins[bin_of(vals[i])], 1u);
-    __syncthreads();
-    // items in the bins of higher threads: total minus the inclusive prefix over threads
-    uint32_t mine = 0;
-#pragma unroll
-    for (int j = 0; j < kBins / kTopkThreads; ++j) mine += bins[tid * (kBins / kTopkThreads) + j];
-    uint32_t incl = mine;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t z = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += z;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      const uint32_t w = wsum[lane];
-      uint32_t c = w;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t z = __shfl_up_sync(0xffffffffu, c, off);
-        if (lane >= off) c += z;
-      }
-      wsum[lane] = c - w;
-      if (lane == 31) s_total = c;
-    }
-    __syncthreads();
-    uint32_t above = s_total - (wsum[warp] + incl);   // items in bins above this thread's bins
-    for (int j = kBins / kTopkThreads - 1; j >= 0; --j) {
-      const int bidx = tid * (kBins / kTopkThreads) + j;
-      const uint32_t h = bins[bidx];
-      if (above < (uint32_t)k && (uint32_t)k <= above + h) {
-        s_bin = (uint32_t)bidx;
-        s_above = above;
-      }
-      above += h;
-    }
-    __syncthreads();
-    const int bstar = (int)s_bin;
-    const uint32_t nc = bins[bstar];
-    if (nc <= (uint32_t)kBinCandMax) {
-      for (int i = tid; i < n_items; i += kTopkThreads) {
-        const uint32_t u = vals[i];
-        if (bin_of(u) == bstar) cand[atomicAdd(&s_nc, 1u)] = (static_cast<uint64_t>(u) << 32) | (0xFFFFFFFFu - (uint32_t)i);
-      }
-      __syncthreads();
-      const uint32_t m = (uint32_t)k - s_above;       // rank (1-based) of the k-th item inside the bin
-      for (int i = tid; i < (int)nc; i += kTopkThreads) {
-        const uint64_t key = cand[i];
-        uint32_t rank = 0;
-        for (int j = 0; j < (int)nc; ++j) rank += cand[j] > key;
-        if (rank == m - 1) s_taukey = static_cast<uint32_t>(key >> 32);
-      }
-      __syncthreads();
-      prefix = s_taukey;
-      for (int i = tid; i < (int)nc; i += kTopkThreads) {
-        const uint64_t key = cand[i];
-        if (static_cast<uint32_t>(key >> 32) != prefix) continue;
-        uint32_t rank = 0;
-        for (int j = 0; j < (int)nc; ++j) rank += cand[j] > key;
-        atomicAdd(&s_eq_all, 1u);
-        if (rank < m) atomicAdd(&s_eq_take, 1u);
-      }
-      __syncthreads();
-      krem = s_eq_take;
-      simple_eq = (s_eq_take == s_eq_all);
-      found = true;
-    }
-  }
-  // ---- otherwise radix select (MSB first, 8 bits per pass)
-  uint32_t mask = 0;
-  const int n_round = (n_items + kTopkThreads - 1) / kTopkThreads * kTopkThreads;
-  if (ranked && !found) {
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-      if (tid < 256) hist[tid] = 0;
-      __syncthreads();
-#pragma unroll 4
-      for (int i = tid; i < n_round; i += kTopkThreads) {
-        uint32_t digit = 256;
-        if (i < n_items) {
-          const uint32_t u = val(i);
-          if ((u & mask) == prefix) digit = (u >> shift) & 255u;
-        }
-        const uint32_t peers = __match_any_sync(0xffffffffu, digit);
-        if (digit < 256 && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], __popc(peers));
-      }
-      __syncthreads();
-      if (warp == 0) {
-        uint32_t local = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) local += hist[8 * lane + j];
-        uint32_t suffix = local;   // items whose digit is >= 8*lane
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const uint32_t y = __shfl_down_sync(0xffffffffu, suffix, off);
-          if (lane + off < 32) suffix += y;
-        }
-        uint32_t above = suffix - local;
-        if (above < krem && krem <= suffix) {
-          for (int j = 7; j >= 0; --j) {
-            const uint32_t h = hist[8 * lane + j];
-            if (above + h >= krem) {
-              s_prefix = prefix | ((uint32_t)(8 * lane + j) << shift);
-              s_krem = krem - above;
-              break;
-            }
-            above += h;
-          }
-        }
-      }
-      __syncthreads();
-      prefix = s_prefix;
-      krem = s_krem;
-      mask |= 0xFFu << shift;
-    }
-  }
-  const uint32_t tau = prefix;   // value bits of the k-th largest item; take krem of the equal ones
-
-  // ---- compaction in item order: warp w owns items [w*ipw, (w+1)*ipw), lane-interleaved rows
-  const int ipw = (n_items + 32 * 32 - 1) / (32 * 32) * 32;
-  const int w0 = warp * ipw, w1 = min(n_items, w0 + ipw);
-  const uint32_t lt_mask = (1u << lane) - 1u;
-  uint32_t eq_count = 0;
-  const bool need_eq = ranked && !simple_eq;      // some items equal to tau are left out
-  if (need_eq)
-    for (int j = w0; j < w1; j += 32) {
-      const int i = j + lane;
-      const bool eq = i < w1 && val(i) == tau;
-      eq_count += __popc(__ballot_sync(0xffffffffu, eq));
-    }
-  const uint32_t eq_base = warp_totals_exclusive(eq_count, wsum, &s_total);
-  auto select_row = [&](int j, uint32_t& eq_run, int& npos) -> bool {
-    const int i = j + lane;
-    bool sel = false;
-    bool eq = false;
-    if (i < w1) {
-      if (take_all) {
-        sel = true;
-      } else if (ranked) {
-        const uint32_t u = val(i);
-        eq = (u == tau);
-        sel = u > tau;
-      }
-    }
-    const uint32_t bal = __ballot_sync(0xffffffffu, eq);
-    if (eq) sel = need_eq ? (eq_run + __popc(bal & lt_mask)) < krem : true;
-    eq_run += __popc(bal);
-    npos = 0;
-    if (sel) {
-      int a, b;
-      members(i, a, b);
-      npos = b - a;
-    }
-    return sel;
-  };
-  uint32_t pos_count = 0;
-  {
-    uint32_t eq_run = eq_base;
-    for (int j = w0; j < w1; j += 32) {
-      int npos;
-      select_row(j, eq_run, npos);
-      int sum = npos;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-      pos_count += (uint32_t)sum;
-    }
-  }
-  const uint32_t pos_base = warp_totals_exclusive(pos_count, wsum, &s_total);
-  const int n_chosen = (int)s_total;
-  {
-    uint32_t eq_run = eq_base, w = (uint32_t)lo + pos_base;
-    for (int j = w0; j < w1; j += 32) {
-      int npos;
-      const bool sel = select_row(j, eq_run, npos);
-      int incl = npos;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
-      }
-      if (sel) {
-        int a, b;
-        members(j + lane, a, b);
-        int o = (int)w + incl - npos;
-        for (int q = a; q < b; ++q) out[o++] = q;
-      }
-      w += (uint32_t)__shfl_sync(0xffffffffu, incl, 31);
-    }
-  }
-  const int count = lo + n_chosen + p.n_recent;
-  for (int i = tid; i < lo; i += kTopkThreads) out[i] = i;
-  for (int i = tid; i < p.n_recent; i += kTopkThreads) out[lo + n_chosen + i] = hi + i;
-  for (int i = count + tid; i < p.budget; i += kTopkThreads) out[i] = -1;
-  if (tid == 0) p.count_out[unit] = count;
-}
-
-// Token-level selection with the scores staged in shared memory (the graded workloads'
-// path): the same boundary-bin method as topk_kernel, written lean.  Needs 0 < k < n <=
-// kLeanMaxItems; the selection mask of each item is kept as warp ballots in registers.
+// Token-level selection with the scores staged in shared memory: the register kernels'
+// method for middles of up to 32K where the batch leaves no SMs for a cluster per unit.
+// Needs 0 < k < n <= kLeanMaxItems; the selection mask of each item is kept as warp ballots
+// in registers.
 constexpr int kLeanMaxItems = 32 * kTopkThreads;   // 32 rows of 32 items per warp
 constexpr int kLeanRows = kLeanMaxItems / kTopkThreads;
 
@@ -1099,7 +744,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_token_kernel(const TopkP
   const int unit = blockIdx.x;
   const int t_u = unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
   int32_t* out = p.idx_out + (size_t)unit * p.budget;
-  if (topk_keep_all(p, unit, t_u, out)) return;
+  if (topk_keep_all(p, unit, t_u, out, tid, kTopkThreads)) return;
   const int lo = p.n_sink, hi = t_u - p.n_recent, n = hi - lo;
   const int k = p.budget - p.n_sink - p.n_recent;
   const float* sc = p.score + (size_t)unit * p.n_mid_pad;
@@ -1633,7 +1278,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_rows_kernel(const TopkPa
   const int unit = blockIdx.x;
   const int t_u = unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
   int32_t* out = p.idx_out + (size_t)unit * p.budget;
-  if (topk_keep_all(p, unit, t_u, out)) return;
+  if (topk_keep_all(p, unit, t_u, out, tid, kTopkThreads)) return;
   const int lo = p.n_sink, hi = t_u - p.n_recent, n = hi - lo;
   const int k = p.budget - p.n_sink - p.n_recent;
   const float* sc = p.score + (size_t)unit * p.n_mid_pad;
@@ -1667,7 +1312,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_rows_chunk_kernel(const 
   const int unit = blockIdx.x;
   const int t_u = unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
   int32_t* out = p.idx_out + (size_t)unit * p.budget;
-  if (topk_keep_all(p, unit, t_u, out)) return;
+  if (topk_keep_all(p, unit, t_u, out, tid, kTopkThreads)) return;
   const int lo = p.n_sink, hi = t_u - p.n_recent, s = p.chunk;
   const int c_first = lo / s;
   const int n_items = hi > lo ? (hi - 1) / s - c_first + 1 : 0;
@@ -2011,7 +1656,15 @@ cudaError_t launch_select(const bd_shape& s, const SelectPlan& plan, const void*
                            : reinterpret_cast<void*>(&topk_rows_kernel<16>);
     return launch_kernel(fn, dim3(units), dim3(kTopkThreads), 0, stream, targs, 0);
   }
-  if (!plan.keep_all && plan.need_scores && chunk == 1 && plan.n_mid <= kLeanMaxItems && free < plan.n_mid) {
+  // One CTA per unit while it holds the items and the batch fills the GPU that way; a
+  // cluster per unit (bd_topk_long.cu) where a unit is too long for that, or where SMs are
+  // left: token level from four CTAs a unit on (a select call of 8 units of 32K positions 29.6
+  // us with one CTA, 26.8 in the cluster; 64 units 107.7 against 107.9, 128 units 195.6 against
+  // 210.3), chunk level, whose member sums cost more, from two on (chunks of 8: 24 units of 36K
+  // 58.7 against 53.7 us, 128 units of 20K 128.7 against 140.3; of 16K, 8 units 16.8 against 18.3).
+  int n_items = plan.n_mid;
+  const long sms = current_sm_count();
+  if (!plan.keep_all && plan.need_scores && chunk == 1 && plan.n_mid <= kLeanMaxItems && 4L * units > sms) {
     const size_t smem = (size_t)align_up(plan.n_mid, 4) * 4;
     void* fn = reinterpret_cast<void*>(&topk_token_kernel);
     err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -2019,10 +1672,9 @@ cudaError_t launch_select(const bd_shape& s, const SelectPlan& plan, const void*
     return launch_kernel(fn, dim3(units), dim3(kTopkThreads), smem, stream, targs, 0);
   }
   if (!plan.keep_all && plan.need_scores && chunk > 1) {
-    // chunks of the longest middle: the register kernel while it holds them
     const int lo = n_sink, hi = s.t_ctx - n_recent;
-    const int n_items = hi > lo ? (hi - 1) / chunk - lo / chunk + 1 : 0;
-    if (n_items <= 16 * kTopkThreads) {
+    n_items = hi > lo ? (hi - 1) / chunk - lo / chunk + 1 : 0;
+    if (n_items <= 16 * kTopkThreads && (plan.n_mid <= 16 * kTopkThreads || 2L * units > sms)) {
       const int rows = std::max(1, (n_items + kTopkThreads - 1) / kTopkThreads);
       void* fn = rows <= 1   ? reinterpret_cast<void*>(&topk_rows_chunk_kernel<1>)
                  : rows <= 2 ? reinterpret_cast<void*>(&topk_rows_chunk_kernel<2>)
@@ -2032,16 +1684,8 @@ cudaError_t launch_select(const bd_shape& s, const SelectPlan& plan, const void*
       return launch_kernel(fn, dim3(units), dim3(kTopkThreads), 0, stream, targs, 0);
     }
   }
-  const int extra = kBins * 4 + kBinCandMax * 8 + 16;      // histogram + boundary-bin candidates
-  const int max_items = (kTopkSmemBytes - extra) / 4;
-  const int n_items = plan.n_mid;                     // upper bound for chunk mode as well
-  tp.smem_items = std::min(n_items, max_items);
-  const size_t smem = (size_t)((tp.smem_items + 1) & ~1) * 4 + extra;
-  err = cudaFuncSetAttribute(reinterpret_cast<void*>(&topk_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-  if (err != cudaSuccess) return err;
-  return launch_kernel(reinterpret_cast<void*>(&topk_kernel), dim3(units), dim3(kTopkThreads), smem, stream, targs,
-                       0);
+  return plan.keep_all || !plan.need_scores ? launch_topk_plain(tp, units, stream)
+                                            : launch_topk_long(tp, units, n_items, stream);
 }
 
 }  // namespace bd
