@@ -127,10 +127,12 @@ void* region(void* ws, int units) { return static_cast<uint8_t*>(ws) + ws_region
 
 bool group_supported_by_draft(int g) { return g >= 1 && g <= 16; }
 
-size_t verify_ws(const bd_shape& s, int n_q, bool with_v, bool* ok) {
-  VerifyPlan vp;
-  *ok = verify_plan(s, n_q, with_v, &vp);
-  return *ok ? ws_region_offset(s.batch * s.h_kv) + verify_partials_bytes(s, vp) : 0;
+// bd_verify_attn without an output: the block's rows are the last n_q positions of a context
+// of t_ctx + n_q
+bd_shape block_context(const bd_shape& s, int n_q) {
+  bd_shape ls = s;
+  ls.t_ctx = s.t_ctx + n_q;
+  return ls;
 }
 
 }  // namespace
@@ -162,10 +164,13 @@ size_t bd_workspace_size(const bd_shape* shape, int op, int budget, int n_q) {
     }
     case BD_OP_VERIFY: {
       if (n_q < 1) return 0;
-      bool ok_v = false, ok_l = false;
-      const size_t a = verify_ws(s, n_q, true, &ok_v);
-      const size_t b = verify_ws(s, n_q, false, &ok_l);
-      if (!ok_v && !ok_l) return 0;
+      VerifyPlan vp;
+      LsePlan lp;
+      const size_t base = ws_region_offset(units);
+      const size_t a = verify_plan(s, n_q, &vp) ? base + verify_partials_bytes(s, vp) : 0;
+      const size_t b = (long long)s.t_ctx + n_q <= s.t_cap && lse_plan(block_context(s, n_q), n_q, &lp)
+                           ? base + lp.part_bytes
+                           : 0;
       return std::max(a, b);
     }
     default:
@@ -265,14 +270,20 @@ int bd_verify_attn(const bd_shape* shape, const void* q, int n_q, const void* k_
   const bool with_v = o_out != nullptr;
   const long long nq_rows = (long long)(s.h_q / s.h_kv) * n_q;
   if (nq_rows > (with_v ? 768 : 128)) return BD_ERR_UNSUPPORTED;
+  const int units = s.batch * s.h_kv;
   VerifyPlan vp;
-  if (!verify_plan(s, n_q, with_v, &vp)) return BD_ERR_UNSUPPORTED;
+  LsePlan lp;
+  if (with_v ? !verify_plan(s, n_q, &vp) : !lse_plan(block_context(s, n_q), n_q, &lp)) return BD_ERR_UNSUPPORTED;
   if (!ws) return BD_ERR_WORKSPACE;
   if (!aligned(ws, 256)) return BD_ERR_MISALIGNED;
-  const int units = s.batch * s.h_kv;
-  if (ws_bytes < ws_region_offset(units) + verify_partials_bytes(s, vp)) return BD_ERR_WORKSPACE;
+  if (ws_bytes < ws_region_offset(units) + (with_v ? verify_partials_bytes(s, vp) : lp.part_bytes))
+    return BD_ERR_WORKSPACE;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (!with_v)
+    return map_cuda(launch_lse(block_context(s, n_q), lp, k_cache, q, n_q, n_q, false, lse_out, region(ws, units),
+                               counters(ws), status_word(ws), st));
   return map_cuda(launch_verify(s, vp, n_q, q, k_cache, v_cache, o_out, lse_out, region(ws, units), counters(ws),
-                                status_word(ws), static_cast<cudaStream_t>(stream)));
+                                status_word(ws), st));
 }
 
 int bd_combine(const float* o_part, const float* lse_part, int n_split, int rows, int head_dim, void* o_out,

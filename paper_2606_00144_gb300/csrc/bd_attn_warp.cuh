@@ -16,12 +16,12 @@
 
 namespace bd {
 
-template <int D, int NT, bool WITH_V>
+template <int D, int NT>
 struct WarpAttn {
   static constexpr int KS = D / 16;
   float m[NT][2];
   float l[NT][2];
-  float o[WITH_V ? KS : 1][NT][4];
+  float o[KS][NT][4];
 
   __device__ __forceinline__ void init() {
 #pragma unroll
@@ -32,7 +32,7 @@ struct WarpAttn {
         l[nt][e] = 0.f;
       }
 #pragma unroll
-      for (int mt = 0; mt < (WITH_V ? KS : 1); ++mt)
+      for (int mt = 0; mt < KS; ++mt)
 #pragma unroll
         for (int c = 0; c < 4; ++c) o[mt][nt][c] = 0.f;
     }
@@ -103,39 +103,37 @@ struct WarpAttn {
         s[nt][2 + e] = p1;
       }
     }
-    if (WITH_V) {
-      if (__any_sync(0xffffffffu, rescale)) {
+    if (__any_sync(0xffffffffu, rescale)) {
 #pragma unroll
-        for (int mt = 0; mt < KS; ++mt)
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            o[mt][nt][0] *= alpha[nt][0];
-            o[mt][nt][1] *= alpha[nt][1];
-            o[mt][nt][2] *= alpha[nt][0];
-            o[mt][nt][3] *= alpha[nt][1];
-          }
-      }
-      uint32_t bp[NT][2], bl[NT][2];
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        uint32_t h0, l0, h1, l1;
-        split_bf16x2(s[nt][0], s[nt][1], h0, l0);
-        split_bf16x2(s[nt][2], s[nt][3], h1, l1);
-        bp[nt][0] = movmatrix_trans(h0);
-        bp[nt][1] = movmatrix_trans(h1);
-        bl[nt][0] = movmatrix_trans(l0);
-        bl[nt][1] = movmatrix_trans(l1);
-      }
-#pragma unroll
-      for (int mt = 0; mt < KS; ++mt) {
-        uint32_t a[4];
-        ldmatrix_x4_trans(a, vbase + sw128_offset(kb + (lane & 7) + 8 * (lane >> 4), 16 * mt + 8 * ((lane >> 3) & 1),
-                                                  half_bytes));
+      for (int mt = 0; mt < KS; ++mt)
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-          mma_16816(o[mt][nt], a, bp[nt][0], bp[nt][1]);
-          mma_16816(o[mt][nt], a, bl[nt][0], bl[nt][1]);
+          o[mt][nt][0] *= alpha[nt][0];
+          o[mt][nt][1] *= alpha[nt][1];
+          o[mt][nt][2] *= alpha[nt][0];
+          o[mt][nt][3] *= alpha[nt][1];
         }
+    }
+    uint32_t bp[NT][2], bl[NT][2];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      uint32_t h0, l0, h1, l1;
+      split_bf16x2(s[nt][0], s[nt][1], h0, l0);
+      split_bf16x2(s[nt][2], s[nt][3], h1, l1);
+      bp[nt][0] = movmatrix_trans(h0);
+      bp[nt][1] = movmatrix_trans(h1);
+      bl[nt][0] = movmatrix_trans(l0);
+      bl[nt][1] = movmatrix_trans(l1);
+    }
+#pragma unroll
+    for (int mt = 0; mt < KS; ++mt) {
+      uint32_t a[4];
+      ldmatrix_x4_trans(a, vbase + sw128_offset(kb + (lane & 7) + 8 * (lane >> 4), 16 * mt + 8 * ((lane >> 3) & 1),
+                                                half_bytes));
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        mma_16816(o[mt][nt], a, bp[nt][0], bp[nt][1]);
+        mma_16816(o[mt][nt], a, bl[nt][0], bl[nt][1]);
       }
     }
   }
@@ -169,21 +167,19 @@ struct WarpAttn {
           l_s[wk * nqc + col] = l[nt][e];
         }
     }
-    if (WITH_V) {
-      constexpr int OP = D + 4;
+    constexpr int OP = D + 4;
 #pragma unroll
-      for (int mt = 0; mt < KS; ++mt)
+    for (int mt = 0; mt < KS; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          const int col = 8 * (col_tile0 + nt) + 2 * tig;
-          const int d0 = 16 * mt + gid;
-          float* base = o_s + (size_t)(wk * nqc + col) * OP;
-          base[d0] = o[mt][nt][0];
-          base[OP + d0] = o[mt][nt][1];
-          base[d0 + 8] = o[mt][nt][2];
-          base[OP + d0 + 8] = o[mt][nt][3];
-        }
-    }
+      for (int nt = 0; nt < NT; ++nt) {
+        const int col = 8 * (col_tile0 + nt) + 2 * tig;
+        const int d0 = 16 * mt + gid;
+        float* base = o_s + (size_t)(wk * nqc + col) * OP;
+        base[d0] = o[mt][nt][0];
+        base[OP + d0] = o[mt][nt][1];
+        base[d0 + 8] = o[mt][nt][2];
+        base[OP + d0 + 8] = o[mt][nt][3];
+      }
   }
 };
 
@@ -191,7 +187,7 @@ struct WarpAttn {
 // WarpAttn::store and emits, per column, a normalised row o (bf16 if o_bf16 else fp32)
 // and lse (natural log).  Out-of-CTA addresses: row r of the output block is
 // o_dst + r*D, lse_dst[r].  Executed by n_threads threads synchronising on bar_id.
-template <int D, int WK, bool WITH_V>
+template <int D, int WK>
 __device__ __forceinline__ void merge_warps_and_store(const float* m_s, const float* l_s, float* f_s,
                                                       const float* o_s, int nqc, int n_cols, float* lse_dst,
                                                       void* o_dst, bool o_bf16, int tid, int n_threads,
@@ -214,7 +210,6 @@ __device__ __forceinline__ void merge_warps_and_store(const float* m_s, const fl
     for (int w = 0; w < WK; ++w) f_s[w * nqc + col] = f[w] * inv;
     if (lse_dst) lse_dst[col] = L > 0.f ? (M + log2f(L)) * kLn2 : -INFINITY;
   }
-  if (!WITH_V || o_dst == nullptr) return;
   named_bar(bar_id, n_threads);
   for (int i = tid; i < n_cols * (D / 2); i += n_threads) {
     const int col = i / (D / 2), d = (i % (D / 2)) * 2;

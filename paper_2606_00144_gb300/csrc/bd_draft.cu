@@ -173,8 +173,8 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
     if (n_tiles > 0) gather(0, 0, 1);
   }
   uint32_t bq[NT][D / 16][2];
-  WarpAttn<D, NT, true>::load_q(bq, p.q + (size_t)unit * p.g * D, p.g, 0, lane);
-  WarpAttn<D, NT, true> wa;
+  WarpAttn<D, NT>::load_q(bq, p.q + (size_t)unit * p.g * D, p.g, 0, lane);
+  WarpAttn<D, NT> wa;
   wa.init();
   for (int t = 0; t < n_tiles; ++t) {
     const int b = dbuf ? (t & 1) : 0;

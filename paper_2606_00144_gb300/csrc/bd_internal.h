@@ -40,16 +40,14 @@ struct VerifyPlan {
   int max_seg;          // most CTAs that share one unit
   int stages;
   size_t smem_bytes;
-  bool with_v;
   bool wide;            // more segments per unit than one staged merge round holds
 };
-bool verify_plan(const bd_shape& s, int n_q, bool with_v, VerifyPlan* plan);
+bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan);
 size_t verify_partials_bytes(const bd_shape& s, const VerifyPlan& plan);
 // q/o/lse as in bd_verify_attn; ws_region points at the op region, counters/status into ws.
 cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, const void* q,
                           const void* k_cache, const void* v_cache, void* o_out, float* lse_out,
-                          void* ws_region, int* counters, int* status, cudaStream_t stream,
-                          int len_offset = 0);
+                          void* ws_region, int* counters, int* status, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------- draft
 struct DraftPlan {
@@ -70,6 +68,21 @@ cudaError_t launch_draft_static(const bd_shape& s, const DraftPlan& plan, const 
                                 const void* v_cache, const int32_t* idx, const int32_t* count, int budget,
                                 int step_j, void* o_out, float* lse_out, cudaStream_t stream);
 
+// ---------------------------------------------------------------------------- row normalisers
+// Softmax normalisers of the last `window` positions' queries over their causal prefixes of a
+// t_ctx-row cache: the selection's self mode, and bd_verify_attn without an output (whose
+// block is the last n_q positions of a context of t_ctx + n_q).
+struct LsePlan {
+  int nq_rows;             // group * window query rows per KV head, at most 128
+  int tiles_per_unit, total_tiles, tiles_per_cta, grid, max_seg;
+  size_t smem_bytes, part_bytes;
+};
+bool lse_plan(const bd_shape& s, int window, LsePlan* plan);
+// len_offset is added to every sequence's length (seq_lens); part: plan.part_bytes of scratch.
+cudaError_t launch_lse(const bd_shape& s, const LsePlan& plan, const void* k_cache, const void* q, int window,
+                       int len_offset, bool window_ready, float* lse_out, void* part, int* counters, int* status,
+                       cudaStream_t stream);
+
 // ---------------------------------------------------------------------------- select
 struct SelectPlan {
   bool keep_all;        // budget >= t_ctx
@@ -83,11 +96,8 @@ struct SelectPlan {
   uint32_t tmem_cols;
   size_t smem_bytes;
   size_t score_bytes, lse_bytes;
-  VerifyPlan lse_plan;  // self mode: window LSE through the verify kernel (lse only)
-  bool self_mode;       // the window LSE can be computed here (one of the two kernels below)
-  bool lse_tc;          // self mode on window_lse_kernel (tcgen05) rather than the verify kernel
-  int lse_tiles_per_unit, lse_total_tiles, lse_tiles_per_cta, lse_grid, lse_max_seg;
-  size_t lse_smem_bytes, lse_part_bytes;
+  bool self_mode;       // the window LSE can be computed here (at most 128 window rows per KV head)
+  LsePlan lse;
 };
 bool select_plan(const bd_shape& s, int window, int budget, int n_sink, int n_recent, int chunk,
                  SelectPlan* plan);

@@ -26,6 +26,7 @@
 //               to 16K positions in registers, topk_token_kernel up to 32K in shared memory;
 //               bd_topk_long.cu spreads longer middles over a cluster.
 #include <algorithm>
+#include <climits>
 
 #include "bd_common.cuh"
 #include "bd_internal.h"
@@ -375,7 +376,7 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
 
 // ============================================================================ window LSE
 //
-// Self mode's normalisers: lse_r = log sum_{k <= p_w} exp(q_r . k_k / sqrt(d)) for the G*W
+// Self mode's normalisers, and bd_verify_attn without an output: lse_r = log sum_{k <= p_w} exp(q_r . k_k / sqrt(d)) for the G*W
 // window rows r = h*W + w of every unit (p_w = t_ctx - W + w).  The contraction of
 // score_kernel with its operands swapped: the unit's window rows are the A operand (M =
 // 128 rows = the TMEM lanes) and a 128-key K tile the B operand (N = 128 columns), so a
@@ -385,6 +386,9 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
 // 4-stage ring) and the unit's rows (two buffers), warp 1 issues the MMAs into four TMEM
 // accumulators, warps 2-9 reduce (two warps per TMEM lane quarter).  A unit split over
 // several CTAs merges the segments' (max, sum) pairs in the CTA that finishes it last.
+// HBM-bound: 268 MB of K (64 units of 16K, 128 rows each) in 51.7 us, 5.2 TB/s; the same rows as
+// an mma.sync verify block without V took 126.9 us, bound by the tensor pipe.  (Skipping the TMEM
+// quarters past nq_rows made the full 128-row case 1 us slower and is left out.)
 struct LseParams {
   const __nv_bfloat16* q_win;   // [units * nq_rows][D] (read by TMA; prefetched through this pointer)
   float* lse;          // [units * nq_rows] natural log
@@ -392,9 +396,11 @@ struct LseParams {
   int* counters;       // [units] arrival counters (left zero)
   int* status;
   int nq_rows, window, t_ctx, tiles_per_unit, total_tiles, tiles_per_cta, max_seg;
+  int settled;         // rows [0, settled) of every unit are older than the preceding kernel
   int window_ready;    // BD_SELECT_WINDOW_READY: the rows may load before the dependency wait
   float scale_log2;
   const int32_t* seq_lens;   // per-sequence context lengths [batch] (RAGGED instance) or null
+  int len_offset;            // added to every length (a verify block ends n_q past its context)
   int h_kv, units;
 };
 constexpr int kLMaxSeg = 8;      // segments of one unit with per-sequence lengths (bounds the partials)
@@ -442,7 +448,7 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
     const int per = (p.units + kLThreads - 1) / kLThreads;
     const int u0 = min(p.units, tid * per), u1 = min(p.units, u0 + per);
     auto tiles_of = [&](int u) {
-      return (unit_context(p.seq_lens, u, p.h_kv, p.t_ctx, nullptr) + kSKeys - 1) / kSKeys;
+      return (unit_context(p.seq_lens, u, p.h_kv, p.t_ctx - p.len_offset, nullptr) + p.len_offset + kSKeys - 1) / kSKeys;
     };
     int sum = 0;
     for (int u = u0; u < u1; ++u) sum += tiles_of(u);
@@ -530,11 +536,16 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
       }
       return __shfl_sync(0xffffffffu, ok, 0);
     };
-    // context K tiles stream before the grid-dependency wait; the window rows after it
-    // (before it as well when the caller says they were written earlier)
-    const int pre = p.window_ready ? 0 : min(n, STAGES);
-    for (int i = 0; i < pre; ++i) issue_k(i);
+    // K tiles of settled rows stream before the grid-dependency wait (with per-sequence lengths
+    // the wait came first); the window rows after it (before it as well when the caller says
+    // they were written earlier)
+    int pre = 0;
     if (!p.window_ready) {
+      auto old_rows = [&](int i) {
+        const int g = first + i;
+        return kSKeys * (g - unit_begin(unit_of(g)) + 1) <= p.settled;
+      };
+      for (; pre < min(n, STAGES) && (RAGGED || old_rows(pre)); ++pre) issue_k(pre);
       if (n > 0)   // the first unit's rows on their way into L2 meanwhile
         prefetch_lines_l2(p.q_win + (size_t)unit_of(first) * p.nq_rows * D, (size_t)p.nq_rows * D * 2, lane, 32);
       grid_dependency_wait();
@@ -621,7 +632,8 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
     for (int i = 0; i < n; ++i) {
       const int g = first + i, unit = unit_of(g), tt = g - unit_begin(unit);
       if (RAGGED && unit != cur_unit) {
-        const int t_u = unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx, tid == 64 ? p.status : nullptr);
+        const int t_u =
+            unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx - p.len_offset, tid == 64 ? p.status : nullptr) + p.len_offset;
         if (t_u < p.window && tid == 64) record_error(p.status, BD_ERR_INVALID_ARG);
         pw = t_u - p.window + row % p.window;
         first_masked = t_u - p.window;
@@ -686,7 +698,7 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
         l = (m == -INFINITY ? 0.f : l * fast_exp2(m - M2)) + (o.x == -INFINITY ? 0.f : o.y * fast_exp2(o.x - M2));
         m = M2;
         if (n_seg == 1) {
-          if (alive && row < p.nq_rows) p.lse[row0 + row] = l > 0.f ? (m + log2f(l)) * kLn2 : -INFINITY;
+          if (alive && row < p.nq_rows) p.lse[row0 + row] = l > 0.f ? fmaf(m, kLn2, logf(l)) : -INFINITY;
         } else if (alive) {
           seg[(size_t)((int)blockIdx.x - c_first) * 128 + row] = make_float2(m, l);
         }
@@ -705,7 +717,7 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
             const float2 ml = __ldcg(&seg[(size_t)k * 128 + row]);
             L += ml.x == -INFINITY ? 0.f : ml.y * fast_exp2(ml.x - M);
           }
-          if (row < p.nq_rows) p.lse[row0 + row] = L > 0.f ? (M + log2f(L)) * kLn2 : -INFINITY;
+          if (row < p.nq_rows) p.lse[row0 + row] = L > 0.f ? fmaf(M, kLn2, logf(L)) : -INFINITY;
           if (row == 0) p.counters[unit] = 0;
         }
       }
@@ -1460,6 +1472,79 @@ uint32_t pow2_at_least(uint32_t x) {
 }
 }  // namespace
 
+bool lse_plan(const bd_shape& s, int window, LsePlan* plan) {
+  *plan = LsePlan{};
+  const long rows = (long)(s.h_q / s.h_kv) * window;
+  if (rows > 128) return false;
+  const long units = (long)s.batch * s.h_kv;
+  const int tpu = (s.t_ctx + kSKeys - 1) / kSKeys;
+  const long total = units * tpu;
+  if (total >= (1L << 31)) return false;
+  int grid = (int)std::max<long>(1, std::min<long>(total, current_sm_count()));
+  int tpc = (int)((total + grid - 1) / grid);
+  int max_seg = 1;
+  if (s.seq_lens) {
+    // the lengths are read on the device: every SM gets a CTA, and the range per CTA is
+    // bounded below so that a unit of tpu tiles spans at most kLMaxSeg ranges
+    grid = current_sm_count();
+    tpc = (tpu + kLMaxSeg - 2) / (kLMaxSeg - 1);
+    max_seg = kLMaxSeg;
+  } else {
+    grid = (int)((total + tpc - 1) / tpc);
+    for (long u = 0; u < units; ++u)
+      max_seg = std::max(max_seg, (int)((u * tpu + tpu - 1) / tpc - (u * tpu) / tpc + 1));
+  }
+  plan->nq_rows = (int)rows;
+  plan->tiles_per_unit = tpu;
+  plan->total_tiles = (int)total;
+  plan->tiles_per_cta = tpc;
+  plan->grid = grid;
+  plan->max_seg = max_seg;
+  plan->smem_bytes = 2048 + (size_t)2 * 128 * s.head_dim * 2 + (size_t)kLStages * kSKeys * s.head_dim * 2 +
+                     2 * 128 * sizeof(float2) + (s.seq_lens ? align_up((size_t)(units + 1) * 4, 16) : 0);
+  plan->part_bytes = max_seg > 1 ? align_up((size_t)units * max_seg * 128 * sizeof(float2), 256) : 0;
+  return plan->smem_bytes <= 227 * 1024;
+}
+
+cudaError_t launch_lse(const bd_shape& s, const LsePlan& plan, const void* k_cache, const void* q, int window,
+                       int len_offset, bool window_ready, float* lse_out, void* part, int* counters, int* status,
+                       cudaStream_t stream) {
+  const int units = s.batch * s.h_kv;
+  CUtensorMap kmap, qmap;
+  cudaError_t err = make_cache_map(&kmap, k_cache, units, s.t_cap, s.t_ctx, s.head_dim, kSKeys);
+  if (err != cudaSuccess) return err;
+  err = make_rows_map(&qmap, q, (long long)units * plan.nq_rows, s.head_dim, 128);
+  if (err != cudaSuccess) return err;
+  LseParams p;
+  p.q_win = static_cast<const __nv_bfloat16*>(q);
+  p.lse = lse_out;
+  p.part = static_cast<float2*>(part);
+  p.counters = counters;
+  p.status = status;
+  p.nq_rows = plan.nq_rows;
+  p.window = window;
+  p.t_ctx = s.t_ctx;
+  p.tiles_per_unit = plan.tiles_per_unit;
+  p.total_tiles = plan.total_tiles;
+  p.tiles_per_cta = plan.tiles_per_cta;
+  p.max_seg = plan.max_seg;
+  p.window_ready = window_ready ? 1 : 0;
+  p.settled = len_offset == 0 ? INT_MAX : s.t_ctx - len_offset;   // a verify block's own rows may be fresh
+  p.seq_lens = s.seq_lens;
+  p.len_offset = len_offset;
+  p.h_kv = s.h_kv;
+  p.units = units;
+  p.scale_log2 = kLog2e / sqrtf((float)s.head_dim);
+  void* fn = s.seq_lens ? (s.head_dim == 64 ? reinterpret_cast<void*>(&window_lse_kernel<64, true>)
+                                            : reinterpret_cast<void*>(&window_lse_kernel<128, true>))
+                        : (s.head_dim == 64 ? reinterpret_cast<void*>(&window_lse_kernel<64, false>)
+                                            : reinterpret_cast<void*>(&window_lse_kernel<128, false>));
+  err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
+  if (err != cudaSuccess) return err;
+  void* args[] = {&p, &kmap, &qmap};
+  return launch_kernel(fn, dim3(plan.grid), dim3(kLThreads), plan.smem_bytes, stream, args, 0);
+}
+
 bool select_plan(const bd_shape& s, int window, int budget, int n_sink, int n_recent, int chunk,
                  SelectPlan* plan) {
   *plan = SelectPlan{};
@@ -1493,55 +1578,12 @@ bool select_plan(const bd_shape& s, int window, int budget, int n_sink, int n_re
   }
   plan->score_bytes = plan->need_scores ? align_up((size_t)units * plan->n_mid_pad * 4, 256) : 0;
   plan->lse_bytes = align_up((size_t)s.batch * s.h_q * window * 4, 256);
-  // self mode's window LSE (carry mode does not need it): window_lse_kernel on the tensor
-  // cores for up to 128 window rows per KV head (with per-sequence lengths a unit spans at
-  // most kLMaxSeg CTA ranges), else the lse-only verify kernel
-  plan->lse_tc = plan->nq_rows <= 128 && (long)units * plan->nq_rows >= 128;
-  if (plan->lse_tc) {
-    const int tpu = (s.t_ctx + kSKeys - 1) / kSKeys;
-    const long total = (long)units * tpu;
-    if (total >= (1L << 31)) return false;
-    int grid = (int)std::max<long>(1, std::min<long>(total, current_sm_count()));
-    int tpc = (int)((total + grid - 1) / grid);
-    int max_seg = 1;
-    if (s.seq_lens) {
-      // the lengths are read on the device: every SM gets a CTA, and the range per CTA is
-      // bounded below so that a unit of tpu tiles spans at most kLMaxSeg ranges
-      grid = current_sm_count();
-      tpc = (tpu + kLMaxSeg - 2) / (kLMaxSeg - 1);
-      max_seg = kLMaxSeg;
-    } else {
-      grid = (int)((total + tpc - 1) / tpc);
-      for (long u = 0; u < units; ++u)
-        max_seg = std::max(max_seg, (int)((u * tpu + tpu - 1) / tpc - (u * tpu) / tpc + 1));
-    }
-    plan->lse_tiles_per_unit = tpu;
-    plan->lse_total_tiles = (int)total;
-    plan->lse_tiles_per_cta = tpc;
-    plan->lse_grid = grid;
-    plan->lse_max_seg = max_seg;
-    plan->lse_smem_bytes = 2048 + (size_t)2 * 128 * s.head_dim * 2 + (size_t)kLStages * kSKeys * s.head_dim * 2 +
-                           2 * 128 * sizeof(float2) + (s.seq_lens ? align_up((size_t)(units + 1) * 4, 16) : 0);
-    plan->lse_part_bytes = max_seg > 1 ? align_up((size_t)units * max_seg * 128 * sizeof(float2), 256) : 0;
-    // a units' table too large for shared memory: the lse-only verify kernel below instead
-    plan->lse_tc = plan->lse_smem_bytes <= 227 * 1024;
-  }
-  if (plan->lse_tc) {
-    plan->self_mode = true;
-  } else {
-    bd_shape ls = s;
-    ls.t_ctx = s.t_ctx - window;
-    plan->self_mode = verify_plan(ls, window, false, &plan->lse_plan);
-  }
+  plan->self_mode = lse_plan(s, window, &plan->lse);   // carry mode does not need it
   return true;
 }
 
-size_t select_region_bytes(const bd_shape& s, const SelectPlan& plan) {
-  if (!plan.self_mode) return plan.score_bytes;
-  bd_shape ls = s;
-  ls.t_ctx = s.t_ctx - plan.nq_rows / std::max(1, s.h_q / s.h_kv);
-  return plan.score_bytes + plan.lse_bytes +
-         (plan.lse_tc ? plan.lse_part_bytes : verify_partials_bytes(ls, plan.lse_plan));
+size_t select_region_bytes(const bd_shape&, const SelectPlan& plan) {
+  return plan.score_bytes + (plan.self_mode ? plan.lse_bytes + plan.lse.part_bytes : 0);
 }
 
 cudaError_t launch_select(const bd_shape& s, const SelectPlan& plan, const void* k_cache,
@@ -1556,44 +1598,8 @@ cudaError_t launch_select(const bd_shape& s, const SelectPlan& plan, const void*
     const float* lse = window_lse;
     if (lse == nullptr) {   // self mode: window LSE over [0, p_w]
       float* lse_buf = reinterpret_cast<float*>(region + plan.score_bytes);
-      if (plan.lse_tc) {
-        CUtensorMap lkmap, lqmap;
-        err = make_cache_map(&lkmap, k_cache, units, s.t_cap, s.t_ctx, s.head_dim, kSKeys);
-        if (err != cudaSuccess) return err;
-        err = make_rows_map(&lqmap, q_window, (long long)units * plan.nq_rows, s.head_dim, 128);
-        if (err != cudaSuccess) return err;
-        LseParams lp;
-        lp.q_win = static_cast<const __nv_bfloat16*>(q_window);
-        lp.lse = lse_buf;
-        lp.part = reinterpret_cast<float2*>(region + plan.score_bytes + plan.lse_bytes);
-        lp.counters = counters;
-        lp.status = status;
-        lp.nq_rows = plan.nq_rows;
-        lp.window = window;
-        lp.t_ctx = s.t_ctx;
-        lp.tiles_per_unit = plan.lse_tiles_per_unit;
-        lp.total_tiles = plan.lse_total_tiles;
-        lp.tiles_per_cta = plan.lse_tiles_per_cta;
-        lp.max_seg = plan.lse_max_seg;
-        lp.window_ready = (flags & BD_SELECT_WINDOW_READY) ? 1 : 0;
-        lp.seq_lens = s.seq_lens;
-        lp.h_kv = s.h_kv;
-        lp.units = units;
-        lp.scale_log2 = kLog2e / sqrtf((float)s.head_dim);
-        void* lfn = s.seq_lens ? (s.head_dim == 64 ? reinterpret_cast<void*>(&window_lse_kernel<64, true>)
-                                                   : reinterpret_cast<void*>(&window_lse_kernel<128, true>))
-                               : (s.head_dim == 64 ? reinterpret_cast<void*>(&window_lse_kernel<64, false>)
-                                                   : reinterpret_cast<void*>(&window_lse_kernel<128, false>));
-        err = cudaFuncSetAttribute(lfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.lse_smem_bytes);
-        if (err != cudaSuccess) return err;
-        void* largs[] = {&lp, &lkmap, &lqmap};
-        err = launch_kernel(lfn, dim3(plan.lse_grid), dim3(kLThreads), plan.lse_smem_bytes, stream, largs, 0);
-      } else {
-        bd_shape ls = s;
-        ls.t_ctx = s.t_ctx - window;
-        err = launch_verify(ls, plan.lse_plan, window, q_window, k_cache, nullptr, nullptr, lse_buf,
-                            region + plan.score_bytes + plan.lse_bytes, counters, status, stream, -window);
-      }
+      err = launch_lse(s, plan.lse, k_cache, q_window, window, 0, (flags & BD_SELECT_WINDOW_READY) != 0, lse_buf,
+                       region + plan.score_bytes + plan.lse_bytes, counters, status, stream);
       if (err != cudaSuccess) return err;
       lse = lse_buf;
     }

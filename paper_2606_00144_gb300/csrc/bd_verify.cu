@@ -1,6 +1,5 @@
-// Verifier block attention (Algorithm 2, Verify) and the window-LSE pass of self-mode
-// selection: n_q queries per head at positions t_ctx .. t_ctx+n_q-1 over keys
-// [0, t_ctx + i] (causal inside the block).
+// Verifier block attention (Algorithm 2, Verify): n_q queries per head at positions
+// t_ctx .. t_ctx+n_q-1 over keys [0, t_ctx + i] (causal inside the block).
 //
 // Persistent, stream-K scheduled: the (unit, 64-key tile) pairs of all (sequence, KV head)
 // units form one list that is cut into contiguous ranges, one per CTA, of equal cost: each
@@ -9,7 +8,7 @@
 // two units; each piece of a unit ("segment") ends in a normalised partial (o, lse), and
 // the last CTA to finish a unit merges its segments (log-sum-exp) into the final bf16
 // output, staging the partials in shared memory with cp.async (one round trip).
-//   warp 4      TMA producer: 64-key K (and V) tiles, 128-byte swizzle, 5-stage ring,
+//   warp 4      TMA producer: 64-key K and V tiles, 128-byte swizzle, 5-stage ring,
 //               streaming straight across segment boundaries.  Context rows [0, t_ctx)
 //               are streamed before the grid-dependency wait (they are not written by
 //               the preceding kernel); the wait comes before the first tile that holds
@@ -44,7 +43,6 @@ struct VerifyParams {
   int* status;
   const int32_t* seq_lens;  // per-sequence context lengths [batch] or null (all t_ctx)
   int h_kv;
-  int len_offset;      // added to every length (the window LSE pass runs at T - W)
   int n_q, nq_rows, t_ctx, tiles_per_unit, total_tiles, max_seg;
   // Query rows of a (sequence, KV head) beyond what one CTA's warps hold are cut into
   // row_chunks chunks of nq_rows rows (the last may hold fewer): a "unit" below is one
@@ -91,14 +89,14 @@ struct VerifyMap {
   __device__ __forceinline__ int owner(int u, int tile) const { return (vbase(u) + a + tile) / vtpc; }
 };
 
-template <int D, int NT, int WQ, bool WITH_V>
+template <int D, int NT, int WQ>
 struct VerifySmem {
   static constexpr int WK = kVConsumers / WQ;
   static constexpr int NQC = 8 * NT * WQ;
   static constexpr uint32_t TILE_BYTES = kVKeys * D * 2;
-  static constexpr uint32_t STAGE_BYTES = (WITH_V ? 2 : 1) * TILE_BYTES;
+  static constexpr uint32_t STAGE_BYTES = 2 * TILE_BYTES;
   static constexpr size_t kStages = (size_t)kVStages * STAGE_BYTES;
-  static constexpr size_t kMerge = (size_t)(3 * WK * NQC) * 4 + (WITH_V ? (size_t)WK * NQC * (D + 4) * 4 : 0);
+  static constexpr size_t kMerge = (size_t)(3 * WK * NQC) * 4 + (size_t)WK * NQC * (D + 4) * 4;
   static constexpr size_t kWeights = (size_t)kVMaxSeg * NQC * 4;
   // layout after the 1 KB barrier block: stages | merge scratch | merge weights
   static constexpr size_t kTotal = 1024 + 1024 + kStages + kMerge + kWeights;
@@ -110,11 +108,11 @@ struct VerifySmem {
 // launched right after, merges them with the whole GPU: a last-CTA merge of ten to twenty
 // parts cost 10-16 us at the end of the kernel.  A separate instance, so that the common
 // case's code (and register allocation) stays as it is.
-template <int D, int NT, int WQ, bool WITH_V, bool WIDE>
+template <int D, int NT, int WQ, bool WIDE>
 __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
                                                            const __grid_constant__ CUtensorMap kmap,
                                                            const __grid_constant__ CUtensorMap vmap) {
-  using L = VerifySmem<D, NT, WQ, WITH_V>;
+  using L = VerifySmem<D, NT, WQ>;
   constexpr int WK = L::WK, SUBS = 4 / WK, NQC = L::NQC;
   constexpr uint32_t HALF_BYTES = kVKeys * 128;
   constexpr int STAGES = kVStages;
@@ -144,8 +142,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
     const int per = (n_units + kVThreads - 1) / kVThreads;
     const int u0 = min(n_units, tid * per), u1 = min(n_units, u0 + per);
     auto span = [&](int u) {
-      const int t_u =
-          max(0, unit_context(p.seq_lens, u / p.row_chunks, p.h_kv, p.t_ctx - p.len_offset, nullptr) + p.len_offset);
+      const int t_u = unit_context(p.seq_lens, u / p.row_chunks, p.h_kv, p.t_ctx, nullptr);
       return (t_u + p.n_q + kVKeys - 1) / kVKeys + p.seg_cost;
     };
     int sum = 0;
@@ -188,7 +185,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
     allow_dependent_launch();
     if (lane == 0) {
       tma_prefetch_map(&kmap);
-      if (WITH_V) tma_prefetch_map(&vmap);
+      tma_prefetch_map(&vmap);
       int issued = 0;
       // with per-sequence lengths any tile may hold some sequence's block rows (written by
       // the preceding kernels): the wait above came before the first load
@@ -213,11 +210,9 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
           mbar_arrive_expect_tx(&full_bar[s], L::STAGE_BYTES);
 #pragma unroll
           for (int h = 0; h < D / 64; ++h) tma_load_3d(st + h * HALF_BYTES, &kmap, &full_bar[s], 64 * h, key0, kv_unit);
-          if (WITH_V) {
 #pragma unroll
-            for (int h = 0; h < D / 64; ++h)
-              tma_load_3d(st + L::TILE_BYTES + h * HALF_BYTES, &vmap, &full_bar[s], 64 * h, key0, kv_unit);
-          }
+          for (int h = 0; h < D / 64; ++h)
+            tma_load_3d(st + L::TILE_BYTES + h * HALF_BYTES, &vmap, &full_bar[s], 64 * h, key0, kv_unit);
           issued = t + 1;
         }
       }
@@ -251,7 +246,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
   // the unit's queries: a chunk of rows of its KV head's block
   auto unit_q = [&](int u, uint32_t (&bq)[NT][D / 16][2]) {
     const int kv = u / p.row_chunks, base = (u - kv * p.row_chunks) * nq;
-    WarpAttn<D, NT, WITH_V>::load_q(bq, p.q + ((size_t)kv * p.rows_total + base) * D, min(nq, p.rows_total - base),
+    WarpAttn<D, NT>::load_q(bq, p.q + ((size_t)kv * p.rows_total + base) * D, min(nq, p.rows_total - base),
                                     wq * NT, lane);
   };
   uint32_t bq[NT][D / 16][2];
@@ -263,8 +258,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
     const int row_base = (unit - kv_unit * p.row_chunks) * nq;   // first row of this chunk
     const int rows = min(nq, p.rows_total - row_base);
     const size_t row0 = (size_t)kv_unit * p.rows_total + row_base;   // its first row in q / o / lse
-    const int t_unit =
-        unit_context(p.seq_lens, kv_unit, p.h_kv, p.t_ctx - p.len_offset, tid == 0 ? p.status : nullptr) + p.len_offset;
+    const int t_unit = unit_context(p.seq_lens, kv_unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -272,7 +266,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
         const int col = 8 * (wq * NT + nt) + 2 * tig + e;
         lim[nt][e] = col < rows ? t_unit + (row_base + col) % p.n_q : -1;
       }
-    WarpAttn<D, NT, WITH_V> wa;
+    WarpAttn<D, NT> wa;
     wa.init();
     for (int tile = tb; tile < te && alive; ++tile, ++t) {
       const int s = t % STAGES;
@@ -308,17 +302,17 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
     const int n_seg = c_last - c_first + 1;
     if (WIDE && c == c_first && tid == 0) p.nseg[unit] = n_seg;
     if (n_seg == 1) {
-      merge_warps_and_store<D, WK, WITH_V>(m_s, l_s, f_s, o_s, NQC, rows, p.lse ? p.lse + row0 : nullptr,
-                                           WITH_V ? static_cast<void*>(p.o + row0 * D) : nullptr, true, tid, NCT, 1);
+      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, rows, p.lse ? p.lse + row0 : nullptr,
+                                           static_cast<void*>(p.o + row0 * D), true, tid, NCT, 1);
     } else if constexpr (WIDE) {
       const size_t slot = (size_t)unit * p.max_seg + (c - c_first);
-      merge_warps_and_store<D, WK, WITH_V>(m_s, l_s, f_s, o_s, NQC, rows, p.lse_part + slot * nq,
-                                           WITH_V ? static_cast<void*>(p.o_part + slot * nq * D) : nullptr, false,
+      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, rows, p.lse_part + slot * nq,
+                                           static_cast<void*>(p.o_part + slot * nq * D), false,
                                            tid, NCT, 1);
     } else {
       const size_t slot = (size_t)unit * p.max_seg + (c - c_first);
-      merge_warps_and_store<D, WK, WITH_V>(m_s, l_s, f_s, o_s, NQC, rows, p.lse_part + slot * nq,
-                                           WITH_V ? static_cast<void*>(p.o_part + slot * nq * D) : nullptr, false,
+      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, rows, p.lse_part + slot * nq,
+                                           static_cast<void*>(p.o_part + slot * nq * D), false,
                                            tid, NCT, 1);
       __threadfence();
       named_bar(1, NCT);
@@ -328,7 +322,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
         __threadfence();
         const size_t base = (size_t)unit * p.max_seg;
         merge_partials<D>(p.o_part + base * nq * D, p.lse_part + base * nq, n_seg, rows, (size_t)nq * D, (size_t)nq,
-                          WITH_V ? p.o + row0 * D : nullptr, p.lse ? p.lse + row0 : nullptr, [](int r) { return r; },
+                          p.o + row0 * D, p.lse ? p.lse + row0 : nullptr, [](int r) { return r; },
                           w_s, tid, NCT, 1, m_s, L::kMerge / 4);
         if (tid == 0) p.counters[unit] = 0;
       }
@@ -428,17 +422,11 @@ struct Variant {
   int nt, wq;
 };
 
-Variant pick_variant(int nq_rows, bool with_v) {
-  if (with_v) {
-    if (nq_rows <= 8) return {1, 1};
-    if (nq_rows <= 24) return {3, 1};
-    if (nq_rows <= 48) return {3, 2};
-    if (nq_rows <= 96) return {3, 4};
-    return {0, 0};
-  }
-  if (nq_rows <= 32) return {4, 1};
-  if (nq_rows <= 64) return {4, 2};
-  if (nq_rows <= 128) return {4, 4};
+Variant pick_variant(int nq_rows) {
+  if (nq_rows <= 8) return {1, 1};
+  if (nq_rows <= 24) return {3, 1};
+  if (nq_rows <= 48) return {3, 2};
+  if (nq_rows <= 96) return {3, 4};
   return {0, 0};
 }
 
@@ -448,23 +436,19 @@ struct KernelInfo {
   size_t merge_floats;   // the staging area a unit's last CTA merges the segments' partials in
 };
 
-template <int D, int NT, int WQ, bool WITH_V, bool WIDE>
+template <int D, int NT, int WQ, bool WIDE>
 KernelInfo info() {
-  return {reinterpret_cast<void*>(&verify_kernel<D, NT, WQ, WITH_V, WIDE>), VerifySmem<D, NT, WQ, WITH_V>::kTotal,
-          VerifySmem<D, NT, WQ, WITH_V>::kMerge / 4};
+  return {reinterpret_cast<void*>(&verify_kernel<D, NT, WQ, WIDE>), VerifySmem<D, NT, WQ>::kTotal,
+          VerifySmem<D, NT, WQ>::kMerge / 4};
 }
 
-KernelInfo select_kernel(int d, int nt, int wq, bool with_v, bool wide) {
-#define BD_VK(DD, N, W, V, X) \
-  if (d == DD && nt == N && wq == W && with_v == V && wide == X) return info<DD, N, W, V, X>();
-  BD_VK(64, 1, 1, true, false) BD_VK(64, 3, 1, true, false) BD_VK(64, 3, 2, true, false) BD_VK(64, 3, 4, true, false)
-  BD_VK(128, 1, 1, true, false) BD_VK(128, 3, 1, true, false) BD_VK(128, 3, 2, true, false)
-  BD_VK(128, 3, 4, true, false)
-  BD_VK(64, 1, 1, true, true) BD_VK(64, 3, 1, true, true) BD_VK(64, 3, 2, true, true) BD_VK(64, 3, 4, true, true)
-  BD_VK(128, 1, 1, true, true) BD_VK(128, 3, 1, true, true) BD_VK(128, 3, 2, true, true)
-  BD_VK(128, 3, 4, true, true)
-  BD_VK(64, 4, 1, false, false) BD_VK(64, 4, 2, false, false) BD_VK(64, 4, 4, false, false)
-  BD_VK(128, 4, 1, false, false) BD_VK(128, 4, 2, false, false) BD_VK(128, 4, 4, false, false)
+KernelInfo select_kernel(int d, int nt, int wq, bool wide) {
+#define BD_VK(DD, N, W, X) \
+  if (d == DD && nt == N && wq == W && wide == X) return info<DD, N, W, X>();
+  BD_VK(64, 1, 1, false) BD_VK(64, 3, 1, false) BD_VK(64, 3, 2, false) BD_VK(64, 3, 4, false)
+  BD_VK(128, 1, 1, false) BD_VK(128, 3, 1, false) BD_VK(128, 3, 2, false) BD_VK(128, 3, 4, false)
+  BD_VK(64, 1, 1, true) BD_VK(64, 3, 1, true) BD_VK(64, 3, 2, true) BD_VK(64, 3, 4, true)
+  BD_VK(128, 1, 1, true) BD_VK(128, 3, 1, true) BD_VK(128, 3, 2, true) BD_VK(128, 3, 4, true)
 #undef BD_VK
   return {nullptr, 0, 0};
 }
@@ -488,23 +472,22 @@ int occupancy(const KernelInfo& k) {
 
 }  // namespace
 
-bool verify_plan(const bd_shape& s, int n_q, bool with_v, VerifyPlan* plan) {
+bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   const int group = s.h_q / s.h_kv;
   const long rows_total = (long)group * n_q;
   // more query rows than one CTA's warps hold (96 with V): chunks of equal size
-  const int chunks = with_v && rows_total > kVMaxRows ? (int)((rows_total + kVMaxRows - 1) / kVMaxRows) : 1;
+  const int chunks = rows_total > kVMaxRows ? (int)((rows_total + kVMaxRows - 1) / kVMaxRows) : 1;
   if (chunks > kVMaxChunks) return false;
   const int nq_rows = (int)((rows_total + chunks - 1) / chunks);
-  const Variant v = pick_variant(nq_rows, with_v);
+  const Variant v = pick_variant(nq_rows);
   if (v.nt == 0) return false;
-  const KernelInfo k = select_kernel(s.head_dim, v.nt, v.wq, with_v, false);
+  const KernelInfo k = select_kernel(s.head_dim, v.nt, v.wq, false);
   if (!k.fn) return false;
   plan->nq_rows = nq_rows;
   plan->rows_total = (int)rows_total;
   plan->row_chunks = chunks;
   plan->nt = v.nt;
   plan->wq = v.wq;
-  plan->with_v = with_v;
   plan->stages = kVStages;
   plan->smem_bytes = k.smem;
   const long n_keys = (long)s.t_ctx + n_q;
@@ -518,7 +501,7 @@ bool verify_plan(const bd_shape& s, int n_q, bool with_v, VerifyPlan* plan) {
   // charge it as virtual tiles at the rate one CTA streams at when every SM streams
   // (~6.5 TB/s over all SMs).  Traced: with 3 us charged, the CTAs holding a boundary ended
   // their last tile ~5 us after the others; swept at 1-12 us, 5 us gave the shortest step.
-  const double tile_bytes = (double)kVKeys * s.head_dim * 2 * (with_v ? 2 : 1);
+  const double tile_bytes = (double)kVKeys * s.head_dim * 2 * 2;
   const double tile_us = tile_bytes / (6.5e6 / (double)std::max(1, current_sm_count()));
   const int a = (int)std::min(16.0, std::max(0.0, 5.0 / tile_us + 0.5));
   const long vtotal = units * (tpu + a);
@@ -548,8 +531,8 @@ bool verify_plan(const bd_shape& s, int n_q, bool with_v, VerifyPlan* plan) {
   }
   // the unit's last CTA merges its segments in one staged round trip while they fit its
   // merge area; more segments take the chunked merge of the wide instance
-  plan->wide = with_v && ((size_t)plan->max_seg * nq_rows * s.head_dim > k.merge_floats ||
-                          (chunks > 1 && plan->max_seg > 1));   // the chunks' units have no arrival counters
+  plan->wide = (size_t)plan->max_seg * nq_rows * s.head_dim > k.merge_floats ||
+               (chunks > 1 && plan->max_seg > 1);   // the chunks' units have no arrival counters
   return true;
 }
 
@@ -562,17 +545,13 @@ size_t verify_partials_bytes(const bd_shape& s, const VerifyPlan& plan) {
 
 cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, const void* q,
                           const void* k_cache, const void* v_cache, void* o_out, float* lse_out,
-                          void* ws_region, int* counters, int* status, cudaStream_t stream, int len_offset) {
+                          void* ws_region, int* counters, int* status, cudaStream_t stream) {
   const int units = s.batch * s.h_kv;
   CUtensorMap kmap, vmap;
   cudaError_t err = make_cache_map(&kmap, k_cache, units, s.t_cap, s.t_ctx + n_q, s.head_dim, kVKeys);
   if (err != cudaSuccess) return err;
-  if (plan.with_v) {
-    err = make_cache_map(&vmap, v_cache, units, s.t_cap, s.t_ctx + n_q, s.head_dim, kVKeys);
-    if (err != cudaSuccess) return err;
-  } else {
-    vmap = kmap;
-  }
+  err = make_cache_map(&vmap, v_cache, units, s.t_cap, s.t_ctx + n_q, s.head_dim, kVKeys);
+  if (err != cudaSuccess) return err;
   VerifyParams p;
   p.q = static_cast<const __nv_bfloat16*>(q);
   p.o = static_cast<__nv_bfloat16*>(o_out);
@@ -590,14 +569,13 @@ cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, co
   p.t_ctx = s.t_ctx;
   p.seq_lens = s.seq_lens;
   p.h_kv = s.h_kv;
-  p.len_offset = len_offset;
   p.tiles_per_unit = plan.tiles_per_unit;
   p.total_tiles = plan.total_tiles;
   p.seg_cost = plan.seg_cost;
   p.vtiles_per_cta = plan.tiles_per_cta;
   p.max_seg = plan.max_seg;
   p.scale_log2 = kLog2e / sqrtf((float)s.head_dim);
-  const KernelInfo k = select_kernel(s.head_dim, plan.nt, plan.wq, plan.with_v, plan.wide);
+  const KernelInfo k = select_kernel(s.head_dim, plan.nt, plan.wq, plan.wide);
   err = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
   if (err != cudaSuccess) return err;
   void* args[] = {&p, &kmap, &vmap};

@@ -72,8 +72,8 @@ class SpecStep:
         self.verify(q_verify, k_cache, v_cache, stream)
 
     def window_lse(self, k_cache, q_win, out=None, stream=None):
-        """LSE of the window queries over their causal prefixes, computed by the verify
-        kernel (what a previous verify / prefill step leaves behind for carry mode).
+        """LSE of the window queries over their causal prefixes, computed by bd_verify_attn
+        without an output (what a previous verify / prefill step leaves behind for carry mode).
 
         The window rows form a verify block that starts W positions before the context's
         end.  With per-sequence lengths, sequence b's rows sit at seq_lens[b] - W ..
