@@ -108,7 +108,8 @@ struct VerifySmem {
 // launched right after, merges them with the whole GPU: a last-CTA merge of ten to twenty
 // parts cost 10-16 us at the end of the kernel.  A separate instance, so that the common
 // case's code (and register allocation) stays as it is.
-template <int D, int NT, int WQ, bool WIDE>
+// UNIFORM: compiled for one shared length only (the other instances decide by p.seq_lens).
+template <int D, int NT, int WQ, bool UNIFORM, bool WIDE>
 __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
                                                            const __grid_constant__ CUtensorMap kmap,
                                                            const __grid_constant__ CUtensorMap vmap) {
@@ -134,7 +135,8 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_units = p.total_tiles / p.tiles_per_unit;
   VerifyMap map{nullptr, p.tiles_per_unit, p.seg_cost, n_units, p.vtiles_per_cta};
-  if (p.seq_lens) {
+  const bool uniform = UNIFORM || p.seq_lens == nullptr;
+  if (!uniform) {
     // per-sequence lengths: every CTA lays out the units' virtual tile spans itself (the
     // lengths may come from the preceding kernel, so after the dependency wait)
     grid_dependency_wait();
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
       int issued = 0;
       // with per-sequence lengths any tile may hold some sequence's block rows (written by
       // the preceding kernels): the wait above came before the first load
-      bool waited = p.seq_lens != nullptr;
+      bool waited = !uniform;
       bool stop = false;
       for (int unit = u_first; unit <= u_last && !stop; ++unit) {
         const int tb = map.first_tile(unit, v0), te = map.end_tile(unit, v1);
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
   }
 
   // -------------------------------------------------------------------- consumers
-  if (!p.seq_lens)   // the first unit's queries on their way into L2 while the predecessor finishes
+  if (uniform)   // the first unit's queries on their way into L2 while the predecessor finishes
     prefetch_lines_l2(p.q + ((size_t)(u_first / p.row_chunks) * p.rows_total + (u_first % p.row_chunks) * p.nq_rows) * D,
                       (size_t)p.nq_rows * D * 2, tid, kVConsumers * 32);
   grid_dependency_wait();                        // the queries come from the preceding kernels
@@ -258,7 +260,8 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
     const int row_base = (unit - kv_unit * p.row_chunks) * nq;   // first row of this chunk
     const int rows = min(nq, p.rows_total - row_base);
     const size_t row0 = (size_t)kv_unit * p.rows_total + row_base;   // its first row in q / o / lse
-    const int t_unit = unit_context(p.seq_lens, kv_unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
+    const int t_unit =
+        UNIFORM ? p.t_ctx : unit_context(p.seq_lens, kv_unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -436,19 +439,20 @@ struct KernelInfo {
   size_t merge_floats;   // the staging area a unit's last CTA merges the segments' partials in
 };
 
-template <int D, int NT, int WQ, bool WIDE>
+template <int D, int NT, int WQ, bool UNIFORM, bool WIDE>
 KernelInfo info() {
-  return {reinterpret_cast<void*>(&verify_kernel<D, NT, WQ, WIDE>), VerifySmem<D, NT, WQ>::kTotal,
+  return {reinterpret_cast<void*>(&verify_kernel<D, NT, WQ, UNIFORM, WIDE>), VerifySmem<D, NT, WQ>::kTotal,
           VerifySmem<D, NT, WQ>::kMerge / 4};
 }
 
-KernelInfo select_kernel(int d, int nt, int wq, bool wide) {
-#define BD_VK(DD, N, W, X) \
-  if (d == DD && nt == N && wq == W && wide == X) return info<DD, N, W, X>();
-  BD_VK(64, 1, 1, false) BD_VK(64, 3, 1, false) BD_VK(64, 3, 2, false) BD_VK(64, 3, 4, false)
-  BD_VK(128, 1, 1, false) BD_VK(128, 3, 1, false) BD_VK(128, 3, 2, false) BD_VK(128, 3, 4, false)
-  BD_VK(64, 1, 1, true) BD_VK(64, 3, 1, true) BD_VK(64, 3, 2, true) BD_VK(64, 3, 4, true)
-  BD_VK(128, 1, 1, true) BD_VK(128, 3, 1, true) BD_VK(128, 3, 2, true) BD_VK(128, 3, 4, true)
+KernelInfo select_kernel(int d, int nt, int wq, bool uniform, bool wide) {
+#define BD_VK(DD, N, W, U)                                                                                    \
+  if (d == DD && nt == N && wq == W && (uniform == U || W > 1))                                                 \
+    return wide ? info<DD, N, W, U, true>() : info<DD, N, W, U, false>();
+  BD_VK(64, 1, 1, true) BD_VK(64, 3, 1, true) BD_VK(64, 1, 1, false) BD_VK(64, 3, 1, false)
+  BD_VK(64, 3, 2, false) BD_VK(64, 3, 4, false)
+  BD_VK(128, 1, 1, true) BD_VK(128, 3, 1, true) BD_VK(128, 1, 1, false) BD_VK(128, 3, 1, false)
+  BD_VK(128, 3, 2, false) BD_VK(128, 3, 4, false)
 #undef BD_VK
   return {nullptr, 0, 0};
 }
@@ -481,7 +485,7 @@ bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   const int nq_rows = (int)((rows_total + chunks - 1) / chunks);
   const Variant v = pick_variant(nq_rows);
   if (v.nt == 0) return false;
-  const KernelInfo k = select_kernel(s.head_dim, v.nt, v.wq, false);
+  const KernelInfo k = select_kernel(s.head_dim, v.nt, v.wq, s.seq_lens == nullptr, false);
   if (!k.fn) return false;
   plan->nq_rows = nq_rows;
   plan->rows_total = (int)rows_total;
@@ -575,7 +579,7 @@ cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, co
   p.vtiles_per_cta = plan.tiles_per_cta;
   p.max_seg = plan.max_seg;
   p.scale_log2 = kLog2e / sqrtf((float)s.head_dim);
-  const KernelInfo k = select_kernel(s.head_dim, plan.nt, plan.wq, plan.wide);
+  const KernelInfo k = select_kernel(s.head_dim, plan.nt, plan.wq, s.seq_lens == nullptr, plan.wide);
   err = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
   if (err != cudaSuccess) return err;
   void* args[] = {&p, &kmap, &vmap};
