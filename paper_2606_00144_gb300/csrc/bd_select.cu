@@ -121,25 +121,28 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
   }
   const int first = blockIdx.x * tpc;
   const int n = max(0, min(tpc, total - first));
-  // (unit, tile within the unit's middle) of tile g of the list
-  auto locate = [&](int g, int& unit, int& tt) {
-    if (!RAGGED) {
-      unit = g / p.tiles_per_unit;
-      tt = g - unit * p.tiles_per_unit;
-      return;
-    }
-    int lo = 0, hi = n_units - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (spref[mid] <= g) lo = mid;
+  // Tile g of the list: its unit and its tile within the unit's middle.  Each role walks the
+  // list with a unit of its own (unit_first to begin with), moved on past unit ends: a division
+  // (or a search of the prefix table) for every tile lengthened the time a K stage is held by
+  // the MMA issuer, which bounds the stream.  64 units of 16K in a whole step 175.1 -> 172.8 us,
+  // 24 ragged units of up to 36K (a select call) 51.0 -> 46.2 us.
+  auto unit_begin = [&](int u) { return RAGGED ? spref[u] : u * p.tiles_per_unit; };
+  int unit_first = 0;
+  if (RAGGED) {
+    int hi = n_units - 1;
+    while (unit_first < hi) {
+      const int mid = (unit_first + hi + 1) >> 1;
+      if (spref[mid] <= first) unit_first = mid;
       else hi = mid - 1;
     }
-    unit = lo;
-    tt = g - spref[lo];
+  } else {
+    unit_first = first / p.tiles_per_unit;
+  }
+  auto locate = [&](int g, int& unit, int& tt) {
+    while (g >= unit_begin(unit + 1)) ++unit;
+    tt = g - unit_begin(unit);
   };
-  auto last_of_unit = [&](int g, int unit) {
-    return RAGGED ? g + 1 == spref[unit + 1] : (g + 1) % p.tiles_per_unit == 0;
-  };
+  auto last_of_unit = [&](int g, int unit) { return g + 1 == unit_begin(unit + 1); };
 
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -175,12 +178,12 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
       tma_prefetch_map(&qmap);
     }
     // K tile i into its ring stage (lane 0; false once a wait gave up)
-    int k_issued = 0;
+    int k_issued = 0, k_unit = unit_first;
     auto issue_k = [&](int i) -> bool {
       bool ok = true;
       if (lane == 0) {
-        int unit, tt;
-        locate(first + i, unit, tt);
+        int tt;
+        locate(first + i, k_unit, tt);
         const int s = i % STAGES;
         if (i >= STAGES) ok = mbar_wait(&empty_bar[s], ((i / STAGES) & 1) ^ 1, p.status, abort_flag);
         if (ok) {
@@ -188,7 +191,7 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
           mbar_arrive_expect_tx(&full_bar[s], KTILE);
           const int key0 = p.n_sink + kSKeys * tt;
 #pragma unroll
-          for (int h = 0; h < D / 64; ++h) tma_load_3d(st + h * KHALF, &kmap, &full_bar[s], 64 * h, key0, unit);
+          for (int h = 0; h < D / 64; ++h) tma_load_3d(st + h * KHALF, &kmap, &full_bar[s], 64 * h, key0, k_unit);
           k_issued = i + 1;
         }
       }
@@ -201,18 +204,14 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
     const int pre = p.window_ready ? 0 : min(n, STAGES);
     for (int i = 0; i < pre; ++i) issue_k(i);
     if (!p.window_ready) {
-      if (n > 0) {   // the first unit's queries on their way into L2 meanwhile
-        int u0, t0;
-        locate(first, u0, t0);
-        prefetch_lines_l2(p.q_win + (size_t)u0 * p.nq_rows * D, (size_t)p.nq_rows * D * 2, lane, 32);
-      }
+      if (n > 0)   // the first unit's queries on their way into L2 meanwhile
+        prefetch_lines_l2(p.q_win + (size_t)unit_first * p.nq_rows * D, (size_t)p.nq_rows * D * 2, lane, 32);
       grid_dependency_wait();
     }
-    int cur_unit = -1, qcount = 0;
+    int cur_unit = -1, qcount = 0, unit = unit_first;
     for (int i = 0; i < n; ++i) {
-      const int g = first + i;
-      int unit, tt;
-      locate(g, unit, tt);
+      int tt;
+      locate(first + i, unit, tt);
       if (unit != cur_unit) {
         const int qs = qcount % NQB;
         bool ok = true;
@@ -245,10 +244,10 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
     allow_dependent_launch();
     if (lane == 0) {
       const uint32_t idesc = umma_idesc_bf16(kSKeys, p.nq_pad);
-      int cur_unit = -1, qcount = 0;
+      int cur_unit = -1, qcount = 0, unit = unit_first;
       for (int i = 0; i < n; ++i) {
         const int g = first + i;
-        int unit, tt;
+        int tt;
         locate(g, unit, tt);
         const bool unit_ends = (i == n - 1) || last_of_unit(g, unit);
         if (unit != cur_unit) {
@@ -284,7 +283,7 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
   } else {
     // ---------------------------------------------------------------- epilogue (2 groups of 4 warps)
     if (!RAGGED && n > 0 && warp == 2)           // the first unit's window LSE into L2 meanwhile
-      prefetch_lines_l2(p.lse_win + (size_t)(first / p.tiles_per_unit) * p.nq_rows, (size_t)p.nq_rows * 4, lane, 32);
+      prefetch_lines_l2(p.lse_win + (size_t)unit_first * p.nq_rows, (size_t)p.nq_rows * 4, lane, 32);
     grid_dependency_wait();                      // the window LSE is carried from earlier kernels
     allow_dependent_launch();
     const int grp = (warp - 2) >> 2;            // group g: warps 2+4g .. 5+4g; tiles i % 4 == g
@@ -294,11 +293,10 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
     int* pw_s = reinterpret_cast<int*>(smem + 1024 + grp * 2304 + 1152);  // [288]
     int win0 = p.t_ctx - p.window;              // position of window row 0 (of the current unit)
     int mid_end = p.mid_end;                    // end of the current unit's middle
-    int cur_unit = -1;
+    int cur_unit = -1, unit = unit_first;
     for (int i = grp; i < n; i += 4) {
-      const int g = first + i;
-      int unit, tt;
-      locate(g, unit, tt);
+      int tt;
+      locate(first + i, unit, tt);
       if (unit != cur_unit) {
         if (RAGGED) {
           const int t_u = unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx, ep_tid == 0 ? p.status : nullptr);
@@ -386,7 +384,7 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
 // 4-stage ring) and the unit's rows (two buffers), warp 1 issues the MMAs into four TMEM
 // accumulators, warps 2-9 reduce (two warps per TMEM lane quarter).  A unit split over
 // several CTAs merges the segments' (max, sum) pairs in the CTA that finishes it last.
-// HBM-bound: 268 MB of K (64 units of 16K, 128 rows each) in 51.7 us, 5.2 TB/s; the same rows as
+// HBM-bound: 268 MB of K (64 units of 16K, 128 rows each) in about 50.8 us, 5.3 TB/s; the same rows as
 // an mma.sync verify block without V took 126.9 us, bound by the tensor pipe.  (Skipping the TMEM
 // quarters past nq_rows made the full 128-row case 1 us slower and is left out.)
 struct LseParams {
@@ -473,18 +471,23 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
   }
   const int first = blockIdx.x * tpc;
   const int n = max(0, min(tpc, total - first));
-  auto unit_of = [&](int g) {
-    if (!RAGGED) return g / tpu;
-    int lo = 0, hi = p.units - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (spref[mid] <= g) lo = mid;
+  auto unit_begin = [&](int u) { return RAGGED ? spref[u] : u * tpu; };
+  auto unit_end = [&](int u) { return unit_begin(u + 1); };
+  // the unit of the range's first tile; each role walks on from it (as in score_kernel)
+  int unit_first = 0;
+  if (RAGGED) {
+    int hi = p.units - 1;
+    while (unit_first < hi) {
+      const int mid = (unit_first + hi + 1) >> 1;
+      if (spref[mid] <= first) unit_first = mid;
       else hi = mid - 1;
     }
-    return lo;
+  } else {
+    unit_first = first / tpu;
+  }
+  auto walk = [&](int g, int& unit) {
+    while (g >= unit_end(unit)) ++unit;
   };
-  auto unit_begin = [&](int u) { return RAGGED ? spref[u] : u * tpu; };
-  auto unit_end = [&](int u) { return RAGGED ? spref[u + 1] : (u + 1) * tpu; };
 
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -519,18 +522,19 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
       tma_prefetch_map(&kmap);
       tma_prefetch_map(&qmap);
     }
-    int k_issued = 0;
+    int k_issued = 0, k_unit = unit_first;
     auto issue_k = [&](int i) -> bool {
       bool ok = true;
       if (lane == 0) {
-        const int g = first + i, unit = unit_of(g), tt = g - unit_begin(unit);
+        walk(first + i, k_unit);
+        const int tt = first + i - unit_begin(k_unit);
         const int s = i % STAGES;
         if (i >= STAGES) ok = mbar_wait(&empty_bar[s], ((i / STAGES) & 1) ^ 1, p.status, abort_flag);
         if (ok) {
           uint8_t* st = kstage + s * KTILE;
           mbar_arrive_expect_tx(&full_bar[s], KTILE);
 #pragma unroll
-          for (int h = 0; h < D / 64; ++h) tma_load_3d(st + h * KHALF, &kmap, &full_bar[s], 64 * h, kSKeys * tt, unit);
+          for (int h = 0; h < D / 64; ++h) tma_load_3d(st + h * KHALF, &kmap, &full_bar[s], 64 * h, kSKeys * tt, k_unit);
           k_issued = i + 1;
         }
       }
@@ -541,18 +545,19 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
     // they were written earlier)
     int pre = 0;
     if (!p.window_ready) {
+      int u = unit_first;
       auto old_rows = [&](int i) {
-        const int g = first + i;
-        return kSKeys * (g - unit_begin(unit_of(g)) + 1) <= p.settled;
+        walk(first + i, u);
+        return kSKeys * (first + i - unit_begin(u) + 1) <= p.settled;
       };
       for (; pre < min(n, STAGES) && (RAGGED || old_rows(pre)); ++pre) issue_k(pre);
       if (n > 0)   // the first unit's rows on their way into L2 meanwhile
-        prefetch_lines_l2(p.q_win + (size_t)unit_of(first) * p.nq_rows * D, (size_t)p.nq_rows * D * 2, lane, 32);
+        prefetch_lines_l2(p.q_win + (size_t)unit_first * p.nq_rows * D, (size_t)p.nq_rows * D * 2, lane, 32);
       grid_dependency_wait();
     }
-    int cur_unit = -1, qcount = 0;
+    int cur_unit = -1, qcount = 0, unit = unit_first;
     for (int i = 0; i < n; ++i) {
-      const int unit = unit_of(first + i);
+      walk(first + i, unit);
       if (unit != cur_unit) {
         const int qs = qcount & 1;
         bool ok = true;
@@ -583,9 +588,10 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
     allow_dependent_launch();
     if (lane == 0) {
       constexpr uint32_t idesc = umma_idesc_bf16(128, kSKeys);
-      int cur_unit = -1, qcount = 0;
+      int cur_unit = -1, qcount = 0, unit = unit_first;
       for (int i = 0; i < n; ++i) {
-        const int g = first + i, unit = unit_of(g);
+        const int g = first + i;
+        walk(g, unit);
         const bool unit_ends = (i == n - 1) || g + 1 == unit_end(unit);
         if (unit != cur_unit) {
           if (!mbar_wait(&qfull_bar[qcount & 1], (qcount >> 1) & 1, p.status, abort_flag)) break;
@@ -624,13 +630,15 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
     const int row = quad * 32 + lane;
     int pw = p.t_ctx - p.window + row % p.window;         // last key the row sees
     int first_masked = p.t_ctx - p.window;                // keys past it are hidden from some row
-    int cur_unit = -1;
+    int cur_unit = -1, unit = unit_first;
     float m = -INFINITY, l = 0.f;                          // log2 units
     // after a wait gives up, a warp keeps walking its tiles without touching TMEM, so that
     // all eight warps still meet at every unit-end barrier
     bool alive = true;
     for (int i = 0; i < n; ++i) {
-      const int g = first + i, unit = unit_of(g), tt = g - unit_begin(unit);
+      const int g = first + i;
+      walk(g, unit);
+      const int tt = g - unit_begin(unit);
       if (RAGGED && unit != cur_unit) {
         const int t_u =
             unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx - p.len_offset, tid == 64 ? p.status : nullptr) + p.len_offset;
