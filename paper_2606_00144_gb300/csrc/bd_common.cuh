@@ -152,6 +152,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
   return mbar_wait_for(bar, parity, status, abort_flag, kWaitLimitNs);
 }
 
+// A whole warp's wait with one answer for all its lanes.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* status, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, abort_flag));
+}
+
 // ---------------------------------------------------------------------------------------
 // TMA (tiled tensor copies global -> shared, completion counted on an mbarrier)
 // ---------------------------------------------------------------------------------------
@@ -258,21 +263,68 @@ __device__ __forceinline__ void tc_fence_before() {
 }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate; one thread issues.
-__device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate) {
+// The MMA issuers run as whole warps in uniform control flow, with one elected lane's
+// predicate on the tcgen05 instructions: descriptors, addresses and loop state then stay in
+// uniform registers.  (As a branch taken by lane 0 alone, issuing an MMA took about 90 cycles,
+// more than the tensor core needs for it.)
+__device__ __forceinline__ uint32_t elect_leader() {
+  uint32_t r;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r;
+}
+// The warp's index as a value the compiler knows to be the same for the whole warp.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
+// Shared-memory matrix descriptors of operands in the 128-byte swizzled layout (8-row x
+// 128-byte atoms): a low word with the address and the leading byte offset, a constant high
+// word (stride byte offset 1024, descriptor version 1, swizzle 128 B).
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+// K-major: atoms stacked every 1024 bytes along M/N (the leading byte offset is unused).
+__device__ __forceinline__ uint32_t desc_k(uint32_t smem_addr) { return ((smem_addr & 0x3FFFFu) >> 4) | (1u << 16); }
+// MN-major: 8 K-rows of 64 MN elements per atom, atoms every 1024 bytes along K and every
+// mn_stride bytes along MN.
+__device__ __forceinline__ uint32_t desc_mn(uint32_t smem_addr, uint32_t mn_stride) {
+  return ((smem_addr & 0x3FFFFu) >> 4) | ((mn_stride >> 4) << 16);
+}
+
+// D[tmem] (+)= A * B^T, bf16 inputs, fp32 accumulate, issued by the lane with lead != 0.  A and
+// B in shared memory (low descriptor words):
+__device__ __forceinline__ void tc_mma_ss(uint32_t lead, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
+                                          uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+      "setp.ne.b32 q, %0, 0;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "mov.b64 da, {%2, %6};\n\t"
+      "mov.b64 db, {%3, %6};\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %4, p;\n\t}" ::"r"(lead),
+      "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi)
       : "memory");
 }
-// Arrive on `bar` once every tcgen05 operation this thread issued so far has completed.
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
+// A in tensor memory:
+__device__ __forceinline__ void tc_mma_ts(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo,
+                                          uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 db;\n\t"
+      "setp.ne.b32 q, %0, 0;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "mov.b64 db, {%3, %6};\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%1], [%2], db, %4, p;\n\t}" ::"r"(lead),
+      "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi)
+      : "memory");
+}
+// Arrive on `bar` once every tcgen05 operation the leader issued so far has completed.
+__device__ __forceinline__ void tc_commit(uint32_t lead, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %0, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n\t}" ::"r"(lead),
+      "r"(smem_u32(bar))
+      : "memory");
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -290,17 +342,6 @@ __device__ __forceinline__ void tc_ld_32cols(uint32_t taddr, float (&v)[32]) {
       : "r"(taddr));
 }
 
-// Shared-memory matrix descriptor for a K-major operand in the 128-byte swizzled layout
-// (8-row x 128-byte atoms, atoms stacked every 1024 bytes along M/N).
-__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((smem_addr & 0x3FFFFu) >> 4);   // start address
-  d |= static_cast<uint64_t>(1) << 16;                        // leading byte offset (unused here)
-  d |= static_cast<uint64_t>(1024 >> 4) << 32;                // stride byte offset: 8 rows * 128 B
-  d |= static_cast<uint64_t>(1) << 46;                        // descriptor version
-  d |= static_cast<uint64_t>(2) << 61;                        // swizzle: 128 B
-  return d;
-}
 // Instruction descriptor: kind::f16 with bf16 A/B, fp32 D, both operands K-major.
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) |

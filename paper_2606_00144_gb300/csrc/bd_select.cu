@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
   uint8_t* qbuf = smem + kSQOffset;                            // NQB x qbytes
   uint8_t* kstage = qbuf + NQB * qbytes;                       // STAGES x KTILE (1024-aligned)
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int n_acc = p.n_acc;
   const int n_units = p.total_tiles / p.tiles_per_unit;
   // per-sequence lengths: every CTA lays out the units' middle tiles itself (prefix table
@@ -240,46 +240,42 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
         mbar_wait(&qfull_bar[q % NQB], (q / NQB) & 1, p.status, nullptr);
     }
   } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer
+    // ---------------------------------------------------------------- MMA issuer (whole warp, see tc_mma_ss)
     allow_dependent_launch();
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(kSKeys, p.nq_pad);
-      int cur_unit = -1, qcount = 0, unit = unit_first;
-      for (int i = 0; i < n; ++i) {
-        const int g = first + i;
-        int tt;
-        locate(g, unit, tt);
-        const bool unit_ends = (i == n - 1) || last_of_unit(g, unit);
-        if (unit != cur_unit) {
-          if (!mbar_wait(&qfull_bar[qcount % NQB], (qcount / NQB) & 1, p.status, abort_flag)) break;
-          cur_unit = unit;
-          ++qcount;
-        }
-        const int qs = (qcount - 1) % NQB;
-        const int s = i % STAGES;
-        if (!mbar_wait(&full_bar[s], (i / STAGES) & 1, p.status, abort_flag)) break;
-        const int acc = i % n_acc;
-        if (i >= n_acc && !mbar_wait(&tempty_bar[acc], ((i / n_acc) & 1) ^ 1, p.status, abort_flag)) break;
-        tc_fence_after();
-        const uint32_t a_base = smem_u32(kstage + s * KTILE);
-        const uint32_t b_base = smem_u32(qbuf + qs * qbytes);
-        const uint32_t b_half = (uint32_t)p.nq_pad * 128;
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * p.acc_stride);
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t koff = (ks & 3) * 32;
-          const uint64_t adesc = umma_desc_sw128(a_base + (ks >> 2) * KHALF + koff);
-          const uint64_t bdesc = umma_desc_sw128(b_base + (ks >> 2) * b_half + koff);
-          tc_mma_bf16(d_tmem, adesc, bdesc, idesc, ks > 0 ? 1u : 0u);
-        }
-        tc_commit(&empty_bar[s]);
-        tc_commit(&tfull_bar[acc]);
-        if (unit_ends) tc_commit(&qempty_bar[qs]);
+    const uint32_t lead = elect_leader();
+    const uint32_t idesc = umma_idesc_bf16(kSKeys, p.nq_pad);
+    const uint32_t b_half = (uint32_t)p.nq_pad * 128;
+    int cur_unit = -1, qcount = 0, unit = unit_first;
+    for (int i = 0; i < n; ++i) {
+      const int g = first + i;
+      int tt;
+      locate(g, unit, tt);
+      const bool unit_ends = (i == n - 1) || last_of_unit(g, unit);
+      if (unit != cur_unit) {
+        if (!mbar_wait_warp(&qfull_bar[qcount % NQB], (qcount / NQB) & 1, p.status, abort_flag)) break;
+        cur_unit = unit;
+        ++qcount;
       }
-      // every MMA this thread issued has completed before TMEM is released
-      tc_commit(drain_bar);
-      mbar_wait(drain_bar, 0, p.status, nullptr);
+      const int qs = (qcount - 1) % NQB;
+      const int s = i % STAGES;
+      const int acc = i % n_acc;
+      if (i >= n_acc && !mbar_wait_warp(&tempty_bar[acc], ((i / n_acc) & 1) ^ 1, p.status, abort_flag)) break;
+      const uint32_t a_lo = desc_k(smem_u32(kstage + s * KTILE));
+      const uint32_t b_lo = desc_k(smem_u32(qbuf + qs * qbytes));
+      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * p.acc_stride);
+      if (!mbar_wait_warp(&full_bar[s], (i / STAGES) & 1, p.status, abort_flag)) break;
+      tc_fence_after();
+#pragma unroll
+      for (int ks = 0; ks < D / 16; ++ks)
+        tc_mma_ss(lead, d_tmem, a_lo + ((ks >> 2) * KHALF + (ks & 3) * 32) / 16,
+                  b_lo + ((ks >> 2) * b_half + (ks & 3) * 32) / 16, idesc, ks > 0 ? 1u : 0u);
+      tc_commit(lead, &empty_bar[s]);
+      tc_commit(lead, &tfull_bar[acc]);
+      if (unit_ends) tc_commit(lead, &qempty_bar[qs]);
     }
+    // every MMA this warp issued has completed before TMEM is released
+    tc_commit(lead, drain_bar);
+    mbar_wait(drain_bar, 0, p.status, nullptr);
   } else {
     // ---------------------------------------------------------------- epilogue (2 groups of 4 warps)
     if (!RAGGED && n > 0 && warp == 2)           // the first unit's window LSE into L2 meanwhile
@@ -435,7 +431,7 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
   float2* ml_s = reinterpret_cast<float2*>(kstage + STAGES * KTILE);   // [2][128] the column halves' (m, l)
   int* spref = reinterpret_cast<int*>(ml_s + 256);                      // [units + 1] (RAGGED)
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int tpu = p.tiles_per_unit;
   int total = p.total_tiles, tpc = p.tiles_per_cta;
   if (RAGGED) {
@@ -584,43 +580,39 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
       for (int q = max(0, qcount - 2); q < qcount; ++q) mbar_wait(&qfull_bar[q & 1], (q >> 1) & 1, p.status, nullptr);
     }
   } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer
+    // ---------------------------------------------------------------- MMA issuer (whole warp, see tc_mma_ss)
     allow_dependent_launch();
-    if (lane == 0) {
-      constexpr uint32_t idesc = umma_idesc_bf16(128, kSKeys);
-      int cur_unit = -1, qcount = 0, unit = unit_first;
-      for (int i = 0; i < n; ++i) {
-        const int g = first + i;
-        walk(g, unit);
-        const bool unit_ends = (i == n - 1) || g + 1 == unit_end(unit);
-        if (unit != cur_unit) {
-          if (!mbar_wait(&qfull_bar[qcount & 1], (qcount >> 1) & 1, p.status, abort_flag)) break;
-          cur_unit = unit;
-          ++qcount;
-        }
-        const int qs = (qcount - 1) & 1;
-        const int s = i % STAGES;
-        if (!mbar_wait(&full_bar[s], (i / STAGES) & 1, p.status, abort_flag)) break;
-        const int acc = i % kLAcc;
-        if (i >= kLAcc && !mbar_wait(&tempty_bar[acc], ((i / kLAcc) & 1) ^ 1, p.status, abort_flag)) break;
-        tc_fence_after();
-        const uint32_t a_base = smem_u32(qbuf + qs * QTILE);
-        const uint32_t b_base = smem_u32(kstage + s * KTILE);
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 128);
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t koff = (ks & 3) * 32;
-          const uint64_t adesc = umma_desc_sw128(a_base + (ks >> 2) * QHALF + koff);
-          const uint64_t bdesc = umma_desc_sw128(b_base + (ks >> 2) * KHALF + koff);
-          tc_mma_bf16(d_tmem, adesc, bdesc, idesc, ks > 0 ? 1u : 0u);
-        }
-        tc_commit(&empty_bar[s]);
-        tc_commit(&tfull_bar[acc]);
-        if (unit_ends) tc_commit(&qempty_bar[qs]);
+    const uint32_t lead = elect_leader();
+    constexpr uint32_t idesc = umma_idesc_bf16(128, kSKeys);
+    int cur_unit = -1, qcount = 0, unit = unit_first;
+    for (int i = 0; i < n; ++i) {
+      const int g = first + i;
+      walk(g, unit);
+      const bool unit_ends = (i == n - 1) || g + 1 == unit_end(unit);
+      if (unit != cur_unit) {
+        if (!mbar_wait_warp(&qfull_bar[qcount & 1], (qcount >> 1) & 1, p.status, abort_flag)) break;
+        cur_unit = unit;
+        ++qcount;
       }
-      tc_commit(drain_bar);
-      mbar_wait(drain_bar, 0, p.status, nullptr);
+      const int qs = (qcount - 1) & 1;
+      const int s = i % STAGES;
+      const int acc = i % kLAcc;
+      if (i >= kLAcc && !mbar_wait_warp(&tempty_bar[acc], ((i / kLAcc) & 1) ^ 1, p.status, abort_flag)) break;
+      const uint32_t a_lo = desc_k(smem_u32(qbuf + qs * QTILE));
+      const uint32_t b_lo = desc_k(smem_u32(kstage + s * KTILE));
+      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 128);
+      if (!mbar_wait_warp(&full_bar[s], (i / STAGES) & 1, p.status, abort_flag)) break;
+      tc_fence_after();
+#pragma unroll
+      for (int ks = 0; ks < D / 16; ++ks)
+        tc_mma_ss(lead, d_tmem, a_lo + ((ks >> 2) * QHALF + (ks & 3) * 32) / 16,
+                  b_lo + ((ks >> 2) * KHALF + (ks & 3) * 32) / 16, idesc, ks > 0 ? 1u : 0u);
+      tc_commit(lead, &empty_bar[s]);
+      tc_commit(lead, &tfull_bar[acc]);
+      if (unit_ends) tc_commit(lead, &qempty_bar[qs]);
     }
+    tc_commit(lead, drain_bar);
+    mbar_wait(drain_bar, 0, p.status, nullptr);
   } else {
     // ---------------------------------------------------------------- epilogue: a row's half per thread
     grid_dependency_wait();
