@@ -167,7 +167,7 @@ size_t bd_workspace_size(const bd_shape* shape, int op, int budget, int n_q) {
       VerifyPlan vp;
       LsePlan lp;
       const size_t base = ws_region_offset(units);
-      const size_t a = verify_plan(s, n_q, &vp) ? base + verify_partials_bytes(s, vp) : 0;
+      const size_t a = verify_plan(s, n_q, &vp) ? base + verify_region_bytes(s, n_q) : 0;
       const size_t b = (long long)s.t_ctx + n_q <= s.t_cap && lse_plan(block_context(s, n_q), n_q, &lp)
                            ? base + lp.part_bytes
                            : 0;

@@ -31,18 +31,20 @@ struct VerifyPlan {
   int nq_rows;          // query rows per unit (a chunk of the group * n_q rows of a KV head)
   int rows_total;       // group * n_q
   int row_chunks;       // chunks of a (sequence, KV head): units = batch * h_kv * row_chunks
-  int nt, wq;           // n-tiles per warp, warp groups along queries
-  int tiles_per_unit;   // 64-key tiles over [0, t_ctx + n_q)
-  int total_tiles;      // over all units
+  int q_tiles;          // M tiles of query rows of verify_tc_kernel, 0: verify_kernel (mma.sync)
+  int nt;               // verify_kernel: n8 tiles of query rows
+  int tiles_per_unit;   // 64-key (verify_tc_kernel: 128-key) tiles over [0, t_ctx + n_q)
   int tiles_per_cta;    // contiguous range of the virtual tile list per CTA
   int seg_cost;         // virtual tiles before each unit's tiles (the cost of starting a unit)
   int grid;
   int max_seg;          // most CTAs that share one unit
-  int stages;
   size_t smem_bytes;
   bool wide;            // more segments per unit than one staged merge round holds
 };
 bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan);
+// What a workspace for blocks of up to n_q queries holds beside its header: a block small enough
+// for verify_kernel may need more partials than a longer one on verify_tc_kernel.
+size_t verify_region_bytes(const bd_shape& s, int n_q);
 size_t verify_partials_bytes(const bd_shape& s, const VerifyPlan& plan);
 // q/o/lse as in bd_verify_attn; ws_region points at the op region, counters/status into ws.
 cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, const void* q,

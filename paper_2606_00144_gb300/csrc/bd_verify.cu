@@ -1,5 +1,6 @@
 // Verifier block attention (Algorithm 2, Verify): n_q queries per head at positions
-// t_ctx .. t_ctx+n_q-1 over keys [0, t_ctx + i] (causal inside the block).
+// t_ctx .. t_ctx+n_q-1 over keys [0, t_ctx + i] (causal inside the block), up to 24 query rows per
+// KV head (more run on verify_tc_kernel, bd_verify_tc.cu); the plan and the launch of both.
 //
 // Persistent, stream-K scheduled: the (unit, 64-key tile) pairs of all (sequence, KV head)
 // units form one list that is cut into contiguous ranges, one per CTA, of equal cost: each
@@ -21,6 +22,7 @@
 #include "bd_attn_warp.cuh"
 #include "bd_common.cuh"
 #include "bd_internal.h"
+#include "bd_verify.cuh"
 
 namespace bd {
 
@@ -28,71 +30,19 @@ constexpr int kVKeys = 64;            // keys per pipeline stage
 constexpr int kVConsumers = 4;        // consumer warps
 constexpr int kVThreads = 160;        // + one producer warp
 constexpr int kVStages = 5;
-constexpr int kVMaxSeg = 33;          // bound on the segments of one unit
-constexpr int kVMaxRows = 96;         // query rows one CTA's consumer warps hold (with V)
-constexpr int kVMaxChunks = 8;        // row chunks of one (sequence, KV head)
+// Query rows of a KV head that verify_kernel takes: three n8 tiles, up to which it streams at
+// memory speed and starts sooner; with more, every tile of keys costs another pass of mma.sync
+// and verify_tc_kernel is faster.  64 units of 16K, both sides measured: 24 rows 86.4 us here, 87.3
+// there; 28 rows 154.5 / 85.4; 84 rows 313.8 / 89.1.  8 units of 4K: 24 rows 10.5 / 11.2, 36 rows
+// 13.4 / 12.6, 84 rows 19.2 / 13.4.
+constexpr int kVMaxRows = 24;
+constexpr int kVTcMaxRows = 256;      // query rows of one unit of verify_tc_kernel: two M tiles
+constexpr int kVMaxChunks = 3;        // row chunks of one (sequence, KV head): 768 query rows in all
 
-struct VerifyParams {
-  const __nv_bfloat16* q;
-  __nv_bfloat16* o;
-  float* lse;
-  float* o_part;       // [units][max_seg][nq_rows][D]
-  float* lse_part;     // [units][max_seg][nq_rows]
-  int* counters;       // [units]
-  int* nseg;           // [units] segments of each unit (wide plans: read by verify_merge_kernel)
-  int* status;
-  const int32_t* seq_lens;  // per-sequence context lengths [batch] or null (all t_ctx)
-  int h_kv;
-  int n_q, nq_rows, t_ctx, tiles_per_unit, total_tiles, max_seg;
-  // Query rows of a (sequence, KV head) beyond what one CTA's warps hold are cut into
-  // row_chunks chunks of nq_rows rows (the last may hold fewer): a "unit" below is one
-  // (sequence, KV head, chunk), and a KV head's chunks are adjacent in the unit list, so
-  // CTAs streaming the same keys run side by side (the second read hits L2).
-  int rows_total;      // group * n_q
-  int row_chunks;
-  int seg_cost;        // virtual tiles charged for each unit a CTA starts (see verify_plan)
-  int vtiles_per_cta;  // contiguous range of the virtual tile list per CTA
-  float scale_log2;    // log2(e) / sqrt(D)
-};
-
-// The global tile list is cut into equal CTA ranges after every unit's tiles are preceded
-// by `seg_cost` virtual tiles: a CTA whose range starts a unit (and so stops to merge one
-// segment and load new queries) receives that many fewer real tiles.
-// The CTA whose range holds real tile g.
-__host__ __device__ __forceinline__ int tile_owner(int g, int tpu, int a, int vtpc) {
-  const int u = g / tpu;
-  return (u * (tpu + a) + a + (g - u * tpu)) / vtpc;
-}
-
-// The same layout seen per unit: unit u spans virtual tiles [vbase(u), vbase(u + 1)), its
-// `a` virtual tiles first, then its real tiles 0 .. tiles(u) - 1; the list is cut into
-// ranges of vtpc virtual tiles, one per CTA.  pref (shared memory, per-sequence lengths)
-// holds vbase(u) for u = 0 .. units; null means every unit has tpu real tiles.
-struct VerifyMap {
-  const int* pref;
-  int tpu, a, units, vtpc;
-  __device__ __forceinline__ int vbase(int u) const { return pref ? pref[u] : u * (tpu + a); }
-  __device__ __forceinline__ int tiles(int u) const { return vbase(u + 1) - vbase(u) - a; }
-  __device__ __forceinline__ int unit_of(int v) const {   // the unit whose span holds v
-    if (!pref) return v / (tpu + a);
-    int lo = 0, hi = units - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (pref[mid] <= v) lo = mid;
-      else hi = mid - 1;
-    }
-    return lo;
-  }
-  // real tiles of unit u inside the virtual range [v0, v1)
-  __device__ __forceinline__ int first_tile(int u, int v0) const { return max(0, v0 - vbase(u) - a); }
-  __device__ __forceinline__ int end_tile(int u, int v1) const { return min(tiles(u), v1 - vbase(u) - a); }
-  __device__ __forceinline__ int owner(int u, int tile) const { return (vbase(u) + a + tile) / vtpc; }
-};
-
-template <int D, int NT, int WQ>
+template <int D, int NT>
 struct VerifySmem {
-  static constexpr int WK = kVConsumers / WQ;
-  static constexpr int NQC = 8 * NT * WQ;
+  static constexpr int WK = kVConsumers;
+  static constexpr int NQC = 8 * NT;
   static constexpr uint32_t TILE_BYTES = kVKeys * D * 2;
   static constexpr uint32_t STAGE_BYTES = 2 * TILE_BYTES;
   static constexpr size_t kStages = (size_t)kVStages * STAGE_BYTES;
@@ -108,15 +58,17 @@ struct VerifySmem {
 // launched right after, merges them with the whole GPU: a last-CTA merge of ten to twenty
 // parts cost 10-16 us at the end of the kernel.  A separate instance, so that the common
 // case's code (and register allocation) stays as it is.
-// UNIFORM: compiled for one shared length only (the other instances decide by p.seq_lens).
-template <int D, int NT, int WQ, bool UNIFORM, bool WIDE>
+// NT: n8 tiles of query rows; SUBS: 16-key sub-tiles of a tile per consumer warp.
+// UNIFORM: one shared context length; the other instances lay out per-sequence lengths.
+template <int D, int NT, int SUBS, bool UNIFORM, bool WIDE>
 __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
                                                            const __grid_constant__ CUtensorMap kmap,
                                                            const __grid_constant__ CUtensorMap vmap) {
-  using L = VerifySmem<D, NT, WQ>;
-  constexpr int WK = L::WK, SUBS = 4 / WK, NQC = L::NQC;
+  using L = VerifySmem<D, NT>;
+  constexpr int WK = L::WK, NQC = L::NQC;
   constexpr uint32_t HALF_BYTES = kVKeys * 128;
   constexpr int STAGES = kVStages;
+  static_assert(16 * SUBS * kVConsumers == kVKeys, "the warps' sub-tiles make up a tile");
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -133,38 +85,13 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
   int* pref = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(w_s) + L::kWeights);   // ragged: [units + 1]
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_units = p.total_tiles / p.tiles_per_unit;
+  const int n_units = p.units;
   VerifyMap map{nullptr, p.tiles_per_unit, p.seg_cost, n_units, p.vtiles_per_cta};
-  const bool uniform = UNIFORM || p.seq_lens == nullptr;
-  if (!uniform) {
+  if (!UNIFORM) {
     // per-sequence lengths: every CTA lays out the units' virtual tile spans itself (the
     // lengths may come from the preceding kernel, so after the dependency wait)
     grid_dependency_wait();
-    int* wtot = reinterpret_cast<int*>(smem + 512);
-    const int per = (n_units + kVThreads - 1) / kVThreads;
-    const int u0 = min(n_units, tid * per), u1 = min(n_units, u0 + per);
-    auto span = [&](int u) {
-      const int t_u = unit_context(p.seq_lens, u / p.row_chunks, p.h_kv, p.t_ctx, nullptr);
-      return (t_u + p.n_q + kVKeys - 1) / kVKeys + p.seg_cost;
-    };
-    int sum = 0;
-    for (int u = u0; u < u1; ++u) sum += span(u);
-    int incl = sum;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, off);
-      if (lane >= off) incl += y;
-    }
-    if (lane == 31) wtot[warp] = incl;
-    __syncthreads();
-    int run = incl - sum;
-    for (int w = 0; w < warp; ++w) run += wtot[w];
-    for (int u = u0; u < u1; ++u) {
-      pref[u] = run;
-      run += span(u);
-    }
-    if (tid == kVThreads - 1) pref[n_units] = run;
-    __syncthreads();
+    lay_out_units<kVThreads, kVKeys>(p, n_units, reinterpret_cast<int*>(smem + 512), pref);
     map.pref = pref;
     map.vtpc = max((pref[n_units] + (int)gridDim.x - 1) / (int)gridDim.x, p.vtiles_per_cta);
   }
@@ -191,11 +118,10 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
       int issued = 0;
       // with per-sequence lengths any tile may hold some sequence's block rows (written by
       // the preceding kernels): the wait above came before the first load
-      bool waited = !uniform;
+      bool waited = !UNIFORM;
       bool stop = false;
       for (int unit = u_first; unit <= u_last && !stop; ++unit) {
         const int tb = map.first_tile(unit, v0), te = map.end_tile(unit, v1);
-        const int kv_unit = unit / p.row_chunks;
         for (int tile = tb; tile < te; ++tile) {
           const int t = issued;
           const int s = t % STAGES;
@@ -211,10 +137,10 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
           uint8_t* st = stage_base + s * L::STAGE_BYTES;
           mbar_arrive_expect_tx(&full_bar[s], L::STAGE_BYTES);
 #pragma unroll
-          for (int h = 0; h < D / 64; ++h) tma_load_3d(st + h * HALF_BYTES, &kmap, &full_bar[s], 64 * h, key0, kv_unit);
+          for (int h = 0; h < D / 64; ++h) tma_load_3d(st + h * HALF_BYTES, &kmap, &full_bar[s], 64 * h, key0, unit);
 #pragma unroll
           for (int h = 0; h < D / 64; ++h)
-            tma_load_3d(st + L::TILE_BYTES + h * HALF_BYTES, &vmap, &full_bar[s], 64 * h, key0, kv_unit);
+            tma_load_3d(st + L::TILE_BYTES + h * HALF_BYTES, &vmap, &full_bar[s], 64 * h, key0, unit);
           issued = t + 1;
         }
       }
@@ -227,14 +153,12 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
   }
 
   // -------------------------------------------------------------------- consumers
-  if (uniform)   // the first unit's queries on their way into L2 while the predecessor finishes
-    prefetch_lines_l2(p.q + ((size_t)(u_first / p.row_chunks) * p.rows_total + (u_first % p.row_chunks) * p.nq_rows) * D,
-                      (size_t)p.nq_rows * D * 2, tid, kVConsumers * 32);
+  if (UNIFORM)   // the first unit's queries on their way into L2 while the predecessor finishes
+    prefetch_lines_l2(p.q + (size_t)u_first * p.nq_rows * D, (size_t)p.nq_rows * D * 2, tid, kVConsumers * 32);
   grid_dependency_wait();                        // the queries come from the preceding kernels
   allow_dependent_launch();
-  const int wq = warp % WQ, wk = warp / WQ;
   const int tig = lane & 3;
-  const int nq = p.nq_rows;                      // rows per unit slot (the chunk size)
+  const int nq = p.nq_rows;                      // query rows of a unit
   constexpr int NCT = kVConsumers * 32;          // consumer threads
   int lim[NT][2];                                // last visible key of each of this thread's columns
 
@@ -245,29 +169,23 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
     while (u <= u_last && map.first_tile(u, v0) >= map.end_tile(u, v1)) ++u;
     return u;
   };
-  // the unit's queries: a chunk of rows of its KV head's block
   auto unit_q = [&](int u, uint32_t (&bq)[NT][D / 16][2]) {
-    const int kv = u / p.row_chunks, base = (u - kv * p.row_chunks) * nq;
-    WarpAttn<D, NT>::load_q(bq, p.q + ((size_t)kv * p.rows_total + base) * D, min(nq, p.rows_total - base),
-                                    wq * NT, lane);
+    WarpAttn<D, NT>::load_q(bq, p.q + (size_t)u * nq * D, nq, 0, lane);
   };
   uint32_t bq[NT][D / 16][2];
   int unit = next_unit(u_first);
   if (unit <= u_last) unit_q(unit, bq);
   for (; unit <= u_last;) {
     const int tb = map.first_tile(unit, v0), te = map.end_tile(unit, v1);
-    const int kv_unit = unit / p.row_chunks;
-    const int row_base = (unit - kv_unit * p.row_chunks) * nq;   // first row of this chunk
-    const int rows = min(nq, p.rows_total - row_base);
-    const size_t row0 = (size_t)kv_unit * p.rows_total + row_base;   // its first row in q / o / lse
+    const size_t row0 = (size_t)unit * nq;       // its first row in q / o / lse
     const int t_unit =
-        UNIFORM ? p.t_ctx : unit_context(p.seq_lens, kv_unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
+        UNIFORM ? p.t_ctx : unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const int col = 8 * (wq * NT + nt) + 2 * tig + e;
-        lim[nt][e] = col < rows ? t_unit + (row_base + col) % p.n_q : -1;
+        const int col = 8 * nt + 2 * tig + e;
+        lim[nt][e] = col < nq ? t_unit + col % p.n_q : -1;
       }
     WarpAttn<D, NT> wa;
     wa.init();
@@ -279,11 +197,10 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
       }
       const uint32_t kbase = smem_u32(stage_base + s * L::STAGE_BYTES);
       const uint32_t vbase = kbase + L::TILE_BYTES;
-      const int key_tile0 = tile * kVKeys;
 #pragma unroll
       for (int sub = 0; sub < SUBS; ++sub) {
-        const int kb = 16 * (wk + WK * sub);
-        const int key_base = key_tile0 + kb;
+        const int kb = 16 * (warp + kVConsumers * sub);
+        const int key_base = tile * kVKeys + kb;
         wa.step(kbase, vbase, HALF_BYTES, kb, bq, p.scale_log2, lane,
                 [&](int ko, int nt, int e) { return key_base + ko <= lim[nt][e]; });
       }
@@ -297,7 +214,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
     wa.finish_rows();
 
     // ---------------------------------------------------------------- end of a segment
-    wa.store(m_s, l_s, o_s, wk, NQC, wq * NT, lane);
+    wa.store(m_s, l_s, o_s, warp, NQC, 0, lane);
     named_bar(1, NCT);
     const int c = blockIdx.x;
     const int c_first = map.owner(unit, 0);
@@ -305,16 +222,16 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
     const int n_seg = c_last - c_first + 1;
     if (WIDE && c == c_first && tid == 0) p.nseg[unit] = n_seg;
     if (n_seg == 1) {
-      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, rows, p.lse ? p.lse + row0 : nullptr,
+      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, nq, p.lse ? p.lse + row0 : nullptr,
                                            static_cast<void*>(p.o + row0 * D), true, tid, NCT, 1);
     } else if constexpr (WIDE) {
       const size_t slot = (size_t)unit * p.max_seg + (c - c_first);
-      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, rows, p.lse_part + slot * nq,
+      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, nq, p.lse_part + slot * nq,
                                            static_cast<void*>(p.o_part + slot * nq * D), false,
                                            tid, NCT, 1);
     } else {
       const size_t slot = (size_t)unit * p.max_seg + (c - c_first);
-      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, rows, p.lse_part + slot * nq,
+      merge_warps_and_store<D, WK>(m_s, l_s, f_s, o_s, NQC, nq, p.lse_part + slot * nq,
                                            static_cast<void*>(p.o_part + slot * nq * D), false,
                                            tid, NCT, 1);
       __threadfence();
@@ -324,7 +241,7 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
       if (*last_flag) {
         __threadfence();
         const size_t base = (size_t)unit * p.max_seg;
-        merge_partials<D>(p.o_part + base * nq * D, p.lse_part + base * nq, n_seg, rows, (size_t)nq * D, (size_t)nq,
+        merge_partials<D>(p.o_part + base * nq * D, p.lse_part + base * nq, n_seg, nq, (size_t)nq * D, (size_t)nq,
                           p.o + row0 * D, p.lse ? p.lse + row0 : nullptr, [](int r) { return r; },
                           w_s, tid, NCT, 1, m_s, L::kMerge / 4);
         if (tid == 0) p.counters[unit] = 0;
@@ -346,8 +263,8 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
 // trips to L2 in all; the groups' sums meet in shared memory.
 template <int D>
 __global__ void __launch_bounds__(128) verify_merge_kernel(const float* o_part, const float* lse_part,
-                                                           const int* nseg, int max_seg, int nq, int rows_total,
-                                                           int row_chunks, __nv_bfloat16* o, float* lse) {
+                                                           const int* nseg, int max_seg, int nq, __nv_bfloat16* o,
+                                                           float* lse) {
   constexpr int Q = D / 4;                 // column quads per row
   constexpr int NG = 128 / Q;              // segment groups
   constexpr int PER = (kVMaxSeg + NG - 1) / NG;
@@ -356,10 +273,9 @@ __global__ void __launch_bounds__(128) verify_merge_kernel(const float* o_part, 
   __shared__ float w[kVMaxSeg];
   __shared__ float4 part[NG][Q];
   const int unit = blockIdx.x, r = blockIdx.y, tid = threadIdx.x;
-  const int kv_unit = unit / row_chunks, row_base = (unit - kv_unit * row_chunks) * nq;
   const int n = min(__ldcg(nseg + unit), kVMaxSeg);
-  if (n <= 1 || row_base + r >= rows_total) return;
-  const size_t orow = (size_t)kv_unit * rows_total + row_base + r;   // the output row
+  if (n <= 1) return;
+  const size_t orow = (size_t)unit * nq + r;        // the output row
   const size_t base = (size_t)unit * max_seg;
   if (tid < 32) {
     const float l0 = tid < n ? __ldcg(lse_part + (base + tid) * nq + r) : -INFINITY;
@@ -421,38 +337,24 @@ __global__ void __launch_bounds__(128) verify_merge_kernel(const float* o_part, 
 
 namespace {
 
-struct Variant {
-  int nt, wq;
-};
-
-Variant pick_variant(int nq_rows) {
-  if (nq_rows <= 8) return {1, 1};
-  if (nq_rows <= 24) return {3, 1};
-  if (nq_rows <= 48) return {3, 2};
-  if (nq_rows <= 96) return {3, 4};
-  return {0, 0};
-}
-
 struct KernelInfo {
   void* fn;
   size_t smem;
   size_t merge_floats;   // the staging area a unit's last CTA merges the segments' partials in
 };
 
-template <int D, int NT, int WQ, bool UNIFORM, bool WIDE>
+template <int D, int NT, bool UNIFORM, bool WIDE>
 KernelInfo info() {
-  return {reinterpret_cast<void*>(&verify_kernel<D, NT, WQ, UNIFORM, WIDE>), VerifySmem<D, NT, WQ>::kTotal,
-          VerifySmem<D, NT, WQ>::kMerge / 4};
+  return {reinterpret_cast<void*>(&verify_kernel<D, NT, kVKeys / (16 * kVConsumers), UNIFORM, WIDE>), VerifySmem<D, NT>::kTotal,
+          VerifySmem<D, NT>::kMerge / 4};
 }
 
-KernelInfo select_kernel(int d, int nt, int wq, bool uniform, bool wide) {
-#define BD_VK(DD, N, W, U)                                                                                    \
-  if (d == DD && nt == N && wq == W && (uniform == U || W > 1))                                                 \
-    return wide ? info<DD, N, W, U, true>() : info<DD, N, W, U, false>();
-  BD_VK(64, 1, 1, true) BD_VK(64, 3, 1, true) BD_VK(64, 1, 1, false) BD_VK(64, 3, 1, false)
-  BD_VK(64, 3, 2, false) BD_VK(64, 3, 4, false)
-  BD_VK(128, 1, 1, true) BD_VK(128, 3, 1, true) BD_VK(128, 1, 1, false) BD_VK(128, 3, 1, false)
-  BD_VK(128, 3, 2, false) BD_VK(128, 3, 4, false)
+KernelInfo select_kernel(int d, int nt, bool uniform, bool wide) {
+#define BD_VK(DD, N, U)                     \
+  if (d == DD && nt == N && uniform == U) \
+    return wide ? info<DD, N, U, true>() : info<DD, N, U, false>();
+  BD_VK(64, 1, true) BD_VK(64, 3, true) BD_VK(64, 1, false) BD_VK(64, 3, false)
+  BD_VK(128, 1, true) BD_VK(128, 3, true) BD_VK(128, 1, false) BD_VK(128, 3, false)
 #undef BD_VK
   return {nullptr, 0, 0};
 }
@@ -479,33 +381,37 @@ int occupancy(const KernelInfo& k) {
 bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   const int group = s.h_q / s.h_kv;
   const long rows_total = (long)group * n_q;
-  // more query rows than one CTA's warps hold (96 with V): chunks of equal size
-  const int chunks = rows_total > kVMaxRows ? (int)((rows_total + kVMaxRows - 1) / kVMaxRows) : 1;
+  const bool tc = rows_total > kVMaxRows;
+  // more query rows than one CTA holds: chunks of equal size
+  const int chunks = tc ? (int)((rows_total + kVTcMaxRows - 1) / kVTcMaxRows) : 1;
   if (chunks > kVMaxChunks) return false;
   const int nq_rows = (int)((rows_total + chunks - 1) / chunks);
-  const Variant v = pick_variant(nq_rows);
-  if (v.nt == 0) return false;
-  const KernelInfo k = select_kernel(s.head_dim, v.nt, v.wq, s.seq_lens == nullptr, false);
-  if (!k.fn) return false;
+  const bool ragged = s.seq_lens != nullptr;
+  const int nt = nq_rows <= 8 ? 1 : 3;
+  const int q_tiles = tc ? (nq_rows > 128 ? 2 : 1) : 0;
+  KernelInfo k = {nullptr, 0, 0};
+  if (!tc) {
+    k = select_kernel(s.head_dim, nt, !ragged, false);
+    if (!k.fn) return false;
+  }
+  const int keys = tc ? kVTcKeys : kVKeys;
   plan->nq_rows = nq_rows;
   plan->rows_total = (int)rows_total;
   plan->row_chunks = chunks;
-  plan->nt = v.nt;
-  plan->wq = v.wq;
-  plan->stages = kVStages;
-  plan->smem_bytes = k.smem;
+  plan->q_tiles = q_tiles;
+  plan->nt = nt;
+  plan->smem_bytes = tc ? verify_tc_smem(s.head_dim, q_tiles) : k.smem;
   const long n_keys = (long)s.t_ctx + n_q;
-  plan->tiles_per_unit = (int)((n_keys + kVKeys - 1) / kVKeys);
+  plan->tiles_per_unit = (int)((n_keys + keys - 1) / keys);
   const long units = (long)s.batch * s.h_kv * chunks;
   const int tpu = plan->tiles_per_unit;
-  const long total = units * tpu;
-  const long ctas = std::max(1, current_sm_count() * occupancy(k));
+  const long ctas = std::max(1, current_sm_count() * (tc ? 1 : occupancy(k)));
   // A unit boundary inside a CTA's range (the segment's merge of the warps' partials, its
   // write, the arrival, the merge by the unit's last CTA) costs about 5 us of streaming time;
   // charge it as virtual tiles at the rate one CTA streams at when every SM streams
   // (~6.5 TB/s over all SMs).  Traced: with 3 us charged, the CTAs holding a boundary ended
   // their last tile ~5 us after the others; swept at 1-12 us, 5 us gave the shortest step.
-  const double tile_bytes = (double)kVKeys * s.head_dim * 2 * 2;
+  const double tile_bytes = (double)keys * s.head_dim * 2 * 2;
   const double tile_us = tile_bytes / (6.5e6 / (double)std::max(1, current_sm_count()));
   const int a = (int)std::min(16.0, std::max(0.0, 5.0 / tile_us + 0.5));
   const long vtotal = units * (tpu + a);
@@ -514,7 +420,6 @@ bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   vtpc = std::max<long>(vtpc, (tpu + a + kVMaxSeg - 2) / (kVMaxSeg - 1));   // <= kVMaxSeg segments
   plan->seg_cost = a;
   plan->tiles_per_cta = (int)vtpc;
-  plan->total_tiles = (int)total;
   plan->grid = (int)((vtotal + vtpc - 1) / vtpc);
   int max_seg = 1;
   for (long u = 0; u < units; ++u) {
@@ -524,7 +429,7 @@ bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   }
   if (max_seg > kVMaxSeg) return false;
   plan->max_seg = max_seg;
-  if (s.seq_lens) {
+  if (ragged) {
     // per-sequence lengths: the kernel cuts the ranges itself over the actual tiles, no
     // shorter than the bound that keeps every unit within kVMaxSeg segments; the units'
     // span table takes (units + 1) ints of shared memory
@@ -535,8 +440,7 @@ bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   }
   // the unit's last CTA merges its segments in one staged round trip while they fit its
   // merge area; more segments take the chunked merge of the wide instance
-  plan->wide = (size_t)plan->max_seg * nq_rows * s.head_dim > k.merge_floats ||
-               (chunks > 1 && plan->max_seg > 1);   // the chunks' units have no arrival counters
+  plan->wide = tc ? plan->max_seg > 1 : (size_t)plan->max_seg * nq_rows * s.head_dim > k.merge_floats;
   return true;
 }
 
@@ -547,14 +451,23 @@ size_t verify_partials_bytes(const bd_shape& s, const VerifyPlan& plan) {
   return align_up(rows * s.head_dim * 4, 256) + align_up(rows * 4, 256) + (plan.wide ? align_up(units * 4, 256) : 0);
 }
 
+size_t verify_region_bytes(const bd_shape& s, int n_q) {
+  VerifyPlan vp;
+  size_t bytes = verify_plan(s, n_q, &vp) ? verify_partials_bytes(s, vp) : 0;
+  const int fewer = kVMaxRows / (s.h_q / s.h_kv);
+  if (fewer >= 1 && fewer < n_q && verify_plan(s, fewer, &vp)) bytes = std::max(bytes, verify_partials_bytes(s, vp));
+  return bytes;
+}
+
 cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, const void* q,
                           const void* k_cache, const void* v_cache, void* o_out, float* lse_out,
                           void* ws_region, int* counters, int* status, cudaStream_t stream) {
   const int units = s.batch * s.h_kv;
+  const int keys = plan.q_tiles ? kVTcKeys : kVKeys;
   CUtensorMap kmap, vmap;
-  cudaError_t err = make_cache_map(&kmap, k_cache, units, s.t_cap, s.t_ctx + n_q, s.head_dim, kVKeys);
+  cudaError_t err = make_cache_map(&kmap, k_cache, units, s.t_cap, s.t_ctx + n_q, s.head_dim, keys);
   if (err != cudaSuccess) return err;
-  err = make_cache_map(&vmap, v_cache, units, s.t_cap, s.t_ctx + n_q, s.head_dim, kVKeys);
+  err = make_cache_map(&vmap, v_cache, units, s.t_cap, s.t_ctx + n_q, s.head_dim, keys);
   if (err != cudaSuccess) return err;
   VerifyParams p;
   p.q = static_cast<const __nv_bfloat16*>(q);
@@ -574,27 +487,35 @@ cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, co
   p.seq_lens = s.seq_lens;
   p.h_kv = s.h_kv;
   p.tiles_per_unit = plan.tiles_per_unit;
-  p.total_tiles = plan.total_tiles;
   p.seg_cost = plan.seg_cost;
   p.vtiles_per_cta = plan.tiles_per_cta;
   p.max_seg = plan.max_seg;
   p.scale_log2 = kLog2e / sqrtf((float)s.head_dim);
-  const KernelInfo k = select_kernel(s.head_dim, plan.nt, plan.wq, s.seq_lens == nullptr, plan.wide);
-  err = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
+  p.units = units * plan.row_chunks;
+  p.tile_rows = plan.q_tiles == 2 ? (plan.nq_rows + 1) / 2 : plan.nq_rows;
+  const void* fn = plan.q_tiles ? verify_tc_fn(s.head_dim, plan.q_tiles, s.seq_lens != nullptr)
+                                : select_kernel(s.head_dim, plan.nt, s.seq_lens == nullptr, plan.wide).fn;
+  err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
   if (err != cudaSuccess) return err;
-  void* args[] = {&p, &kmap, &vmap};
-  err = launch_kernel(k.fn, dim3(plan.grid), dim3(kVThreads), plan.smem_bytes, stream, args, 0);
+  CUtensorMap qmap;
+  if (plan.q_tiles) {
+    err = make_rows_map(&qmap, q, (long long)units * plan.rows_total, s.head_dim, 128);
+    if (err != cudaSuccess) return err;
+  }
+  void* args[] = {&p, &kmap, &vmap, &qmap};   // (verify_kernel takes the first three)
+  err = launch_kernel(fn, dim3(plan.grid), dim3(plan.q_tiles ? kVTcThreads : kVThreads), plan.smem_bytes, stream, args, 0);
   if (err != cudaSuccess || !plan.wide) return err;
+  if (plan.q_tiles) return launch_verify_tc_merge(s.head_dim, p.units, p, stream);
   const float* op = p.o_part;
   const float* lp = p.lse_part;
   const int* ns = p.nseg;
-  int max_seg = plan.max_seg, nq = plan.nq_rows, rows_total = plan.rows_total, chunks = plan.row_chunks;
+  int max_seg = plan.max_seg, nq = plan.nq_rows;
   __nv_bfloat16* o = p.o;
   float* l = p.lse;
-  void* margs[] = {&op, &lp, &ns, &max_seg, &nq, &rows_total, &chunks, &o, &l};
+  void* margs[] = {&op, &lp, &ns, &max_seg, &nq, &o, &l};
   void* mfn = s.head_dim == 64 ? reinterpret_cast<void*>(&verify_merge_kernel<64>)
                                : reinterpret_cast<void*>(&verify_merge_kernel<128>);
-  return launch_kernel(mfn, dim3(units * plan.row_chunks, plan.nq_rows), dim3(128), 0, stream, margs, 0);
+  return launch_kernel(mfn, dim3(units, plan.nq_rows), dim3(128), 0, stream, margs, 0);
 }
 
 }  // namespace bd
