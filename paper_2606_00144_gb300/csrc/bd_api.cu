@@ -159,8 +159,8 @@ size_t bd_workspace_size(const bd_shape* shape, int op, int budget, int n_q) {
     case BD_OP_DRAFT: {
       if (n_q < 1 || budget < 1) return 0;
       DraftPlan dp;
-      if (!draft_plan(s, budget, n_q, &dp)) return 0;
-      return ws_region_offset(units) + draft_partials_bytes(s, dp);
+      if (!draft_plan(s, budget, n_q, SIZE_MAX, &dp)) return 0;
+      return ws_region_offset(units) + draft_region_bytes(s);
     }
     case BD_OP_VERIFY: {
       if (n_q < 1) return 0;
@@ -221,11 +221,12 @@ int bd_draft_attn(const bd_shape* shape, const void* q, const void* k_cache, con
   if (flags & ~BD_DRAFT_VIEW_READY) return BD_ERR_INVALID_ARG;
   if (!group_supported_by_draft(s.h_q / s.h_kv)) return BD_ERR_UNSUPPORTED;
   DraftPlan dp;
-  if (!draft_plan(s, budget, step_j + 1, &dp)) return BD_ERR_UNSUPPORTED;
+  const int units = s.batch * s.h_kv;
+  const size_t base = ws_region_offset(units);
+  if (!draft_plan(s, budget, step_j + 1, ws_bytes > base ? ws_bytes - base : 0, &dp)) return BD_ERR_UNSUPPORTED;
   if (!ws) return BD_ERR_WORKSPACE;
   if (!aligned(ws, 256)) return BD_ERR_MISALIGNED;
-  const int units = s.batch * s.h_kv;
-  if (ws_bytes < ws_region_offset(units) + draft_partials_bytes(s, dp)) return BD_ERR_WORKSPACE;
+  if (ws_bytes < base) return BD_ERR_WORKSPACE;
   return map_cuda(launch_draft(s, dp, q, k_cache, v_cache, idx, count, budget, step_j, flags, o_out, lse_out,
                                region(ws, units), counters(ws), status_word(ws), static_cast<cudaStream_t>(stream)));
 }
@@ -247,9 +248,10 @@ int bd_draft_attn_static(const bd_shape* shape, const void* q, const void* k_cac
   if (budget < 1 || step_j < 0 || (long long)s.t_ctx + step_j >= s.t_cap) return BD_ERR_INVALID_ARG;
   if (!group_supported_by_draft(s.h_q / s.h_kv)) return BD_ERR_UNSUPPORTED;
   DraftPlan dp;
-  if (!draft_plan(s, budget, step_j + 1, &dp)) return BD_ERR_UNSUPPORTED;
   const int units = s.batch * s.h_kv;
-  if (ws_region_offset(units) + draft_partials_bytes(s, dp) > draft_static_scratch_bytes()) return BD_ERR_WORKSPACE;
+  // (every call shares the array, so no partials in it: one cluster per unit)
+  if (!draft_plan(s, budget, step_j + 1, 0, &dp)) return BD_ERR_UNSUPPORTED;
+  if (ws_region_offset(units) > draft_static_scratch_bytes()) return BD_ERR_WORKSPACE;
   return map_cuda(launch_draft_static(s, dp, q, k_cache, v_cache, idx, count, budget, step_j, o_out, lse_out,
                                       static_cast<cudaStream_t>(stream)));
 }

@@ -14,6 +14,8 @@
 //      cluster's rank-0 CTA (distributed shared memory); after one cluster barrier rank 0
 //      merges them (log-sum-exp) from its own shared memory and writes the bf16 output:
 //      no global partials, fences or atomics.
+// Long views of few units are spread over several clusters per unit (LONG instances, chosen by
+// draft_plan); those leave a partial each in global memory and the unit's last one merges them.
 // Launched with programmatic dependent launch: the grid-dependency wait is the first thing
 // a CTA does, except with BD_DRAFT_VIEW_READY, where the selected rows (and the unit's
 // context length) are read and gathered first and only the queries and the drafted rows
@@ -22,6 +24,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "bd_attn_warp.cuh"
 #include "bd_common.cuh"
@@ -31,10 +34,10 @@ namespace cg = cooperative_groups;
 
 namespace bd {
 
-constexpr int kDRows = 80;        // rows per shared-memory tile: 5 sub-tiles of 16, one per warp
-constexpr int kDWarps = kDRows / 16;
-constexpr int kDThreads = 32 * kDWarps;
-constexpr int kDMaxCluster = 8;   // CTAs per (sequence, KV head): the portable cluster size
+constexpr int kDRows = 80;        // rows per shared-memory tile: sub-tiles of 16, one per warp
+constexpr int kDLongRows = 160;   // the same for long slices (LONG instances)
+constexpr int kDMaxCluster = 8;   // CTAs of a cluster: the portable cluster size
+constexpr int kDMaxParts = 8;     // clusters per unit
 
 struct DraftParams {
   const __nv_bfloat16* q;      // [units * g][D]
@@ -55,12 +58,22 @@ struct DraftParams {
   float scale_log2;
 };
 
-template <int D, int G>
+// (A type of its own: with these fields in DraftParams the short instances were compiled differently,
+// 3% slower on views of 64 units x 2K rows.)
+struct DraftLongParams : DraftParams {
+  int n_clusters;              // clusters of n_split CTAs per unit
+  float* o_part;               // [units][n_clusters][g][D + 4]: a cluster's normalised rows, their lse
+  int* counters;               // [units] arrivals of the unit's clusters (left zero)
+};
+
+template <int D, int G, bool LONG>
 struct DraftSmem {
+  static constexpr int ROWS = LONG ? kDLongRows : kDRows;
+  static constexpr int WARPS = ROWS / 16, THREADS = 32 * WARPS;
   static constexpr int NQC = 8 * ((G + 7) / 8);   // query columns: the group in n8 tiles
-  static constexpr uint32_t TILE_BYTES = kDRows * D * 2;
+  static constexpr uint32_t TILE_BYTES = ROWS * D * 2;
   static constexpr uint32_t STAGE_BYTES = 2 * TILE_BYTES;                 // K and V
-  static constexpr size_t kMerge = (size_t)(3 * kDWarps * NQC) * 4 + (size_t)kDWarps * NQC * (D + 4) * 4;
+  static constexpr size_t kMerge = (size_t)(3 * WARPS * NQC) * 4 + (size_t)WARPS * NQC * (D + 4) * 4;
   // one CTA's partial in rank 0: G rows of D floats, then G lse padded to 16 bytes
   static constexpr int kSlot = G * D + ((G + 3) & ~3);
   // stages (the warp-merge scratch reuses them) | rowpos [pos_slots] (the row of every
@@ -71,15 +84,66 @@ struct DraftSmem {
   }
 };
 
-template <int D, int G>
-__global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
-  using L = DraftSmem<D, G>;
+// The unit's last cluster to arrive merges the clusters' partials: part [n][g_rows][D + 4] (a
+// normalised row, its lse), by the threads of its leading CTA.  Every part of an item is requested at
+// once.  `arrived` is left at zero.
+template <int D, int THREADS>
+__device__ __forceinline__ void merge_clusters(const float* part, int n, int g_rows, int* arrived, __nv_bfloat16* o,
+                                               float* lse, int tid) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(arrived, 1) == n - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = tid; i < g_rows * (D / 4); i += THREADS) {
+    const int g = i / (D / 4), d = (i % (D / 4)) * 4;
+    float lr[kDMaxParts];
+    float4 v[kDMaxParts];
+    float mx = -INFINITY;
+#pragma unroll
+    for (int r = 0; r < kDMaxParts; ++r) {
+      const float* row = part + (size_t)(r * g_rows + g) * (D + 4);
+      lr[r] = r < n ? __ldcg(row + D) : -INFINITY;
+      v[r] = r < n ? __ldcg(reinterpret_cast<const float4*>(row + d)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int r = 0; r < kDMaxParts; ++r) mx = fmaxf(mx, lr[r]);
+    float tot = 0.f;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int r = 0; r < kDMaxParts; ++r) {
+      const float w = lr[r] == -INFINITY ? 0.f : fast_exp2((lr[r] - mx) * kLog2e);
+      tot += w;
+      a.x += w * v[r].x;
+      a.y += w * v[r].y;
+      a.z += w * v[r].z;
+      a.w += w * v[r].w;
+    }
+    const float inv = tot > 0.f ? 1.f / tot : 0.f;
+    *reinterpret_cast<uint2*>(o + (size_t)g * D + d) =
+        make_uint2(pack_bf16x2(a.x * inv, a.y * inv), pack_bf16x2(a.z * inv, a.w * inv));
+    if (d == 0 && lse) lse[g] = mx == -INFINITY ? -INFINITY : mx + logf(tot);
+  }
+  if (tid == 0) *arrived = 0;
+}
+
+// LONG: the instance for views that leave a CTA many tiles: twice the warps and rows a tile (an
+// iteration is a chain of latencies, about 1.2 us whatever the tile holds), one CTA per SM, and
+// several clusters per unit where SMs are left.  4 units of 8K rows (d 128, groups of 8): 16.2 us
+// a pass in 32 CTAs of five warps, 12.5 with ten, 7.7 over all SMs; traced, 1 us of that is the
+// dependency wait, 2.5 the tiles, 2 the cluster's merge and 2 the clusters'.
+template <int D, int G, bool LONG>
+__global__ void __launch_bounds__(DraftSmem<D, G, LONG>::THREADS) draft_kernel(const std::conditional_t<LONG, DraftLongParams, DraftParams> p) {
+  using L = DraftSmem<D, G, LONG>;
+  constexpr int kRows = L::ROWS, kWarps = L::WARPS, kThreads = L::THREADS;
   constexpr int NT = (G + 7) / 8, NQC = L::NQC;   // the group's query heads in n8 tiles
-  constexpr uint32_t HALF_BYTES = kDRows * 128;
+  constexpr uint32_t HALF_BYTES = kRows * 128;
   constexpr int CH = D / 8;                    // 16-byte chunks per row
   const bool early = (p.flags & BD_DRAFT_VIEW_READY) != 0;
   // the pass's queries (read after the wait below) on their way into L2 meanwhile
-  prefetch_lines_l2(p.q + (size_t)blockIdx.y * p.g * D, (size_t)p.g * D * 2, threadIdx.x, kDThreads);
+  prefetch_lines_l2(p.q + (size_t)blockIdx.y * p.g * D, (size_t)p.g * D * 2, threadIdx.x, kThreads);
   if (!early) {
     grid_dependency_wait();
     allow_dependent_launch();
@@ -94,9 +158,9 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
   int* rowpos = reinterpret_cast<int*>(smem + stage_bytes);               // [pos_slots]
   float* parts = reinterpret_cast<float*>(rowpos + p.pos_slots);          // [C][kSlot]
   float* m_s = reinterpret_cast<float*>(stage);                           // warp-merge scratch
-  float* l_s = m_s + kDWarps * NQC;
-  float* f_s = l_s + kDWarps * NQC;
-  float* o_s = f_s + kDWarps * NQC;
+  float* l_s = m_s + kWarps * NQC;
+  float* f_s = l_s + kWarps * NQC;
+  float* o_s = f_s + kWarps * NQC;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int split = blockIdx.x, unit = blockIdx.y;
@@ -106,7 +170,7 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
   const int e_begin = split * p.rows_per_split;
   // count and the first tile's indices in flight together
   int idx_pref = -1;
-  if (tid < kDRows) {
+  if (tid < kRows) {
     const int e = e_begin + tid;
     if (e < p.budget && tid < p.rows_per_split) idx_pref = __ldg(iunit + e);
   }
@@ -120,7 +184,7 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
   const int t_unit = unit_context(p.seq_lens, unit, p.h_kv, p.t_ctx, tid == 0 ? p.status : nullptr);
   const int n_entries = cnt + p.step_j + 1;
   const int e_end = min(e_begin + p.rows_per_split, n_entries);
-  const int n_tiles = e_end > e_begin ? (e_end - e_begin + kDRows - 1) / kDRows : 0;
+  const int n_tiles = e_end > e_begin ? (e_end - e_begin + kRows - 1) / kRows : 0;
   const __nv_bfloat16* kunit = p.k + (size_t)unit * p.t_cap * D;
   const __nv_bfloat16* vunit = p.v + (size_t)unit * p.t_cap * D;
 
@@ -135,21 +199,21 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
   // the row of every entry of the slice, up front: tile 0 from the prefetched indices, the
   // later tiles' loads all in flight together (no index round trip between tiles)
   auto set_all_rows = [&]() {
-    if (tid < kDRows) {
+    if (tid < kRows) {
       const int e = e_begin + tid;
       rowpos[tid] = e < e_end ? position(e, idx_pref) : -1;
     }
-    for (int e = e_begin + kDRows + tid; e < e_end; e += kDThreads)
+    for (int e = e_begin + kRows + tid; e < e_end; e += kThreads)
       rowpos[e - e_begin] = position(e, e < cnt ? __ldg(iunit + e) : 0);
   };
   // part 0: context rows (and zero fill), part 1: drafted rows (t_ctx and later), part 2: all
   auto gather = [&](int tile, int b, int part) {
-    const int nrows = min(kDRows, e_end - (e_begin + tile * kDRows));
+    const int nrows = min(kRows, e_end - (e_begin + tile * kRows));
     uint8_t* kt = stage + b * L::STAGE_BYTES;
     uint8_t* vt = kt + L::TILE_BYTES;
-    for (int c = tid; c < kDRows * CH; c += kDThreads) {
+    for (int c = tid; c < kRows * CH; c += kThreads) {
       const int r = c / CH, ch = c % CH;
-      const int pos = rowpos[tile * kDRows + r];
+      const int pos = rowpos[tile * kRows + r];
       const bool live = r < nrows && pos >= 0;   // others zero-filled (0 * garbage could be NaN in P V)
       const bool drafted = live && pos >= t_unit;
       if ((part == 0 && drafted) || (part == 1 && !drafted)) continue;
@@ -185,9 +249,9 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
       cp_async_wait<0>();
     }
     __syncthreads();
-    const int nrows = min(kDRows, e_end - (e_begin + t * kDRows));
+    const int nrows = min(kRows, e_end - (e_begin + t * kRows));
     const uint32_t kbase = smem_u32(stage + b * L::STAGE_BYTES);
-    const int* rp = rowpos + t * kDRows;
+    const int* rp = rowpos + t * kRows;
     if (16 * warp < nrows) {
       const int kb = 16 * warp;
       wa.step(kbase, kbase + L::TILE_BYTES, HALF_BYTES, kb, bq, p.scale_log2, lane, [&](int ko, int, int) {
@@ -203,8 +267,8 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
   __syncthreads();
   const size_t row0 = (size_t)unit * p.g;
   if (p.n_split == 1) {
-    merge_warps_flat<D, kDWarps, true>(m_s, l_s, o_s, NQC, p.g, p.lse ? p.lse + row0 : nullptr, p.o + row0 * D, tid,
-                                       kDThreads);
+    merge_warps_flat<D, kWarps, true>(m_s, l_s, o_s, NQC, p.g, p.lse ? p.lse + row0 : nullptr, p.o + row0 * D, tid,
+                                       kThreads);
     return;
   }
   // ---------------------------------------------------------------- cluster merge (DSMEM)
@@ -214,11 +278,11 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
   const int rank = (int)cluster.block_rank();
   float* slot = cluster.map_shared_rank(parts, 0) + (size_t)rank * SLOT;   // in rank 0
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // every CTA is running
-  merge_warps_flat<D, kDWarps, false>(m_s, l_s, o_s, NQC, G, slot + G * D, slot, tid, kDThreads);
+  merge_warps_flat<D, kWarps, false>(m_s, l_s, o_s, NQC, G, slot + G * D, slot, tid, kThreads);
   cluster.sync();                                  // all partials have landed in rank 0
   if (rank != 0) return;
   // each thread: four output columns of one head, its merge weights derived in place
-  for (int i = tid; i < p.g * (D / 4); i += kDThreads) {
+  for (int i = tid; i < p.g * (D / 4); i += kThreads) {
     const int g = i / (D / 4), d = (i % (D / 4)) * 4;
     float lr[kDMaxCluster];
     float mx = -INFINITY;
@@ -242,11 +306,24 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
       }
     }
     const float inv = tot > 0.f ? 1.f / tot : 0.f;
+    if constexpr (LONG) {
+      if (p.n_clusters > 1) {
+        float* own = p.o_part + (((size_t)unit * p.n_clusters + split / C) * p.g + g) * (D + 4);
+        *reinterpret_cast<float4*>(own + d) = make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv);
+        if (d == 0) own[D] = mx == -INFINITY ? -INFINITY : mx + logf(tot);
+        continue;
+      }
+    }
     uint2 packed;
     packed.x = pack_bf16x2(a.x * inv, a.y * inv);
     packed.y = pack_bf16x2(a.z * inv, a.w * inv);
     *reinterpret_cast<uint2*>(p.o + (row0 + g) * D + d) = packed;
     if (d == 0 && p.lse) p.lse[row0 + g] = mx == -INFINITY ? -INFINITY : mx + logf(tot);
+  }
+  if constexpr (LONG) {
+    if (p.n_clusters > 1)
+      merge_clusters<D, kThreads>(p.o_part + (size_t)unit * p.n_clusters * p.g * (D + 4), p.n_clusters, p.g,
+                                  &p.counters[unit], p.o + row0 * D, p.lse ? p.lse + row0 : nullptr, tid);
   }
 }
 
@@ -254,17 +331,20 @@ __global__ void __launch_bounds__(kDThreads) draft_kernel(const DraftParams p) {
 
 namespace {
 using DraftFn = void*;
-DraftFn pick(int d, int g) {
-#define BD_DK(DD, GG) \
-  if (d == DD && g == GG) return reinterpret_cast<void*>(&draft_kernel<DD, GG>);
+DraftFn pick(int d, int g, bool longs) {
+#define BD_DK(DD, GG)                                                              \
+  if (d == DD && g == GG)                                                          \
+    return longs ? reinterpret_cast<void*>(&draft_kernel<DD, GG, true>) : reinterpret_cast<void*>(&draft_kernel<DD, GG, false>);
   BD_DK(64, 1) BD_DK(64, 2) BD_DK(64, 4) BD_DK(64, 8) BD_DK(64, 16)
   BD_DK(128, 1) BD_DK(128, 2) BD_DK(128, 4) BD_DK(128, 8) BD_DK(128, 16)
 #undef BD_DK
   return nullptr;
 }
-size_t smem_bytes(int d, int g, int n_stage, int cluster, int pos_slots) {
-#define BD_DS(DD, GG) \
-  if (d == DD && g == GG) return DraftSmem<DD, GG>::bytes(n_stage, cluster, pos_slots);
+size_t smem_bytes(int d, int g, bool longs, int n_stage, int cluster, int pos_slots) {
+#define BD_DS(DD, GG)                                                         \
+  if (d == DD && g == GG)                                                     \
+    return longs ? DraftSmem<DD, GG, true>::bytes(n_stage, cluster, pos_slots) \
+                 : DraftSmem<DD, GG, false>::bytes(n_stage, cluster, pos_slots);
   BD_DS(64, 1) BD_DS(64, 2) BD_DS(64, 4) BD_DS(64, 8) BD_DS(64, 16)
   BD_DS(128, 1) BD_DS(128, 2) BD_DS(128, 4) BD_DS(128, 8) BD_DS(128, 16)
 #undef BD_DS
@@ -277,21 +357,75 @@ size_t smem_bytes(int d, int g, int n_stage, int cluster, int pos_slots) {
 // loop gains more from overlapping its own gathers than from a single wave); a CTA of two
 // tiles in a larger grid relies on its co-resident CTAs to hide its gathers.
 static int draft_stages(const DraftPlan& plan, long units) {
+  if (plan.longs) return 2;
   return (plan.rows_per_split > kDRows && units * plan.n_split <= 2L * current_sm_count()) ||
                  plan.rows_per_split > 2 * kDRows
              ? 2
              : 1;
 }
 // Entries of the CTA's row table: its slice rounded up to whole tiles.
-static int draft_pos_slots(const DraftPlan& plan) { return (plan.rows_per_split + kDRows - 1) / kDRows * kDRows; }
+static int draft_pos_slots(const DraftPlan& plan) {
+  const int rows = plan.longs ? kDLongRows : kDRows;
+  return (plan.rows_per_split + rows - 1) / rows * rows;
+}
 
 // The kernel instance whose n8 query tiles hold a group of g query heads (g <= 16: one
 // tile up to 8, two beyond).
 int draft_group_instance(int g) { return g <= 1 ? 1 : g <= 2 ? 2 : g <= 4 ? 4 : g <= 8 ? 8 : 16; }
 
-bool draft_plan(const bd_shape& s, int budget, int n_steps, DraftPlan* plan) {
+// Clusters of c CTAs of a LONG instance (one CTA per SM) that the device holds at once.
+static long long_clusters(int d, int g_kernel, int c) {
+  static thread_local int cache_dev = -1;
+  static thread_local int cache[kDMaxCluster + 1];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return current_sm_count() / c;
+  }
+  if (dev != cache_dev) {
+    for (int& n : cache) n = -1;
+    cache_dev = dev;
+  }
+  if (cache[c] < 0) {
+    void* fn = pick(d, g_kernel, true);
+    const size_t smem = 200 * 1024;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(2 * kDLongRows);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)c;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      n = current_sm_count() / c;
+    }
+    cache[c] = n;
+  }
+  return cache[c];
+}
+
+// One cluster per unit merges in shared memory; several leave a partial each.
+size_t draft_partials_bytes(const bd_shape& s, const DraftPlan& plan) {
+  if (plan.n_clusters == 1) return 0;
+  return align_up((size_t)s.batch * s.h_q * plan.n_clusters * (s.head_dim + 4) * sizeof(float), 256);
+}
+
+// Room for the most clusters that any budget or pass of the shape is given.
+size_t draft_region_bytes(const bd_shape& s) {
+  DraftPlan most = {};
+  most.n_clusters = kDMaxParts;
+  return 6L * s.batch * s.h_kv <= current_sm_count() ? draft_partials_bytes(s, most) : 0;
+}
+
+bool draft_plan(const bd_shape& s, int budget, int n_steps, size_t room, DraftPlan* plan) {
   const int g = s.h_q / s.h_kv;
-  if (g < 1 || g > 16 || !pick(s.head_dim, draft_group_instance(g))) return false;
+  if (g < 1 || g > 16 || !pick(s.head_dim, draft_group_instance(g), false)) return false;
   const long entries = (long)budget + n_steps;
   // one tile per CTA up to a cluster of 8, but no more CTAs than one wave holds at the
   // occupancy the slice's stage count gives (three single-stage or two double-buffered
@@ -309,22 +443,44 @@ bool draft_plan(const bd_shape& s, int budget, int n_steps, DraftPlan* plan) {
   if (rows_per_split > (1L << 24)) return false;
   plan->rows_per_split = (int)rows_per_split;
   plan->n_split = n_split;
+  plan->n_clusters = 1;
+  plan->longs = false;
   // the row table of a CTA's slice sits in shared memory beside its tiles
   const int g_kernel = draft_group_instance(g);
-  return smem_bytes(s.head_dim, g_kernel, draft_stages(*plan, units), n_split, draft_pos_slots(*plan)) <=
+  // A LONG instance where its estimate is the shorter: a fixed cost, one per tile a CTA walks
+  // (both fitted to passes of 4 units of 1K to 8K rows), one where clusters meet in memory.  Per pass,
+  // d 128, short / LONG measured: 4 units of 1K rows 5.1 / 4.8 us, 2K 7.2 / 5.8, 8K 16.2 / 7.7; 8 units of
+  // 8K 16.4 / 10.6; 16 units of 1K 5.4 / 6.2 (stays short), 4K 11.9 / 10.6; 64 units of 2K 13.5 / 13.5 (the
+  // L2's rate; stays short).  Clusters of two CTAs gained nothing.
+  double best_us = 3.1 + 1.0 * ((rows_per_split + kDRows - 1) / kDRows);
+  for (int c = kDMaxCluster; c >= 3; --c) {
+    const long cap = long_clusters(s.head_dim, g_kernel, c);
+    for (int k = 1; k <= kDMaxParts && units * k <= cap; ++k) {
+      const long rps = (entries + c * k - 1) / (c * k);
+      const double us = 3.0 + 1.33 * ((rps + kDLongRows - 1) / kDLongRows) + (k > 1 ? 2.05 : 0.0);
+      if (us >= best_us) continue;
+      DraftPlan lp;
+      lp.n_split = c;
+      lp.n_clusters = k;
+      lp.rows_per_split = (int)rps;
+      lp.longs = true;
+      if (draft_partials_bytes(s, lp) > room ||
+          smem_bytes(s.head_dim, g_kernel, true, 2, c, draft_pos_slots(lp)) > 227 * 1024)
+        continue;
+      *plan = lp;
+      best_us = us;
+    }
+  }
+  return smem_bytes(s.head_dim, g_kernel, plan->longs, draft_stages(*plan, units), plan->n_split, draft_pos_slots(*plan)) <=
          227 * 1024;
 }
-
-size_t draft_partials_bytes(const bd_shape&, const DraftPlan&) { return 0; }   // merged in the cluster
 
 cudaError_t launch_draft(const bd_shape& s, const DraftPlan& plan, const void* q, const void* k_cache,
                          const void* v_cache, const int32_t* idx, const int32_t* count, int budget,
                          int step_j, unsigned flags, void* o_out, float* lse_out, void* ws_region,
                          int* counters, int* status, cudaStream_t stream) {
-  (void)ws_region;
-  (void)counters;
   const int units = s.batch * s.h_kv;
-  DraftParams p;
+  DraftLongParams p;             // (a short instance takes its first part)
   p.q = static_cast<const __nv_bfloat16*>(q);
   p.k = static_cast<const __nv_bfloat16*>(k_cache);
   p.v = static_cast<const __nv_bfloat16*>(v_cache);
@@ -341,6 +497,9 @@ cudaError_t launch_draft(const bd_shape& s, const DraftPlan& plan, const void* q
   p.t_cap = s.t_cap;
   p.n_split = plan.n_split;
   p.rows_per_split = plan.rows_per_split;
+  p.n_clusters = plan.n_clusters;
+  p.o_part = static_cast<float*>(ws_region);
+  p.counters = counters;
   p.n_stage = draft_stages(plan, units);
   p.pos_slots = draft_pos_slots(plan);
   p.flags = flags;
@@ -348,14 +507,15 @@ cudaError_t launch_draft(const bd_shape& s, const DraftPlan& plan, const void* q
   const int g = s.h_q / s.h_kv;
   const int g_kernel = draft_group_instance(g);
   p.g = g;
-  void* fn = pick(s.head_dim, g_kernel);
-  const size_t smem = smem_bytes(s.head_dim, g_kernel, p.n_stage, plan.n_split, p.pos_slots);
+  void* fn = pick(s.head_dim, g_kernel, plan.longs);
+  const size_t smem = smem_bytes(s.head_dim, g_kernel, plan.longs, p.n_stage, plan.n_split, p.pos_slots);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
 
   void* args[] = {&p};
-  return launch_kernel(fn, dim3(plan.n_split, units), dim3(kDThreads), smem, stream, args,
+  return launch_kernel(fn, dim3(plan.n_split * plan.n_clusters, units),
+                       dim3(2 * (plan.longs ? kDLongRows : kDRows)), smem, stream, args,
                        plan.n_split > 1 ? plan.n_split : 0);
 }
 

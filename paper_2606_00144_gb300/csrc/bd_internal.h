@@ -53,10 +53,14 @@ cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, co
 
 // ---------------------------------------------------------------------------- draft
 struct DraftPlan {
-  int n_split;
-  int rows_per_split;
+  int n_split;          // CTAs of a cluster
+  int n_clusters;       // clusters of a (sequence, KV head)
+  int rows_per_split;   // entries of a CTA's slice
+  bool longs;           // the LONG kernel instance
 };
-bool draft_plan(const bd_shape& s, int budget, int n_steps, DraftPlan* plan);
+// room: bytes of the op region; a plan that needs more is not made.
+bool draft_plan(const bd_shape& s, int budget, int n_steps, size_t room, DraftPlan* plan);
+size_t draft_region_bytes(const bd_shape& s);
 size_t draft_partials_bytes(const bd_shape& s, const DraftPlan& plan);
 cudaError_t launch_draft(const bd_shape& s, const DraftPlan& plan, const void* q, const void* k_cache,
                          const void* v_cache, const int32_t* idx, const int32_t* count, int budget,
