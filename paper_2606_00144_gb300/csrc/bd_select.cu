@@ -36,7 +36,7 @@ namespace bd {
 
 constexpr int kSKeys = 128;          // keys per tile (UMMA M)
 constexpr int kSThreads = 576;       // producer, MMA, 4 x 4 epilogue warps
-constexpr int kMaxAcc = 4;           // TMEM accumulators (<= 512 columns)
+constexpr int kSGroups = 4;          // epilogue groups of four warps
 constexpr int kSQOffset = 12288;     // shared-memory offset of the window-query tiles
 
 struct ScoreParams {
@@ -67,9 +67,12 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem);
   uint64_t* empty_bar = full_bar + STAGES;
-  uint64_t* tfull_bar = empty_bar + STAGES;        // [kMaxAcc]
-  uint64_t* tempty_bar = tfull_bar + kMaxAcc;      // [kMaxAcc]
-  uint64_t* qfull_bar = tempty_bar + kMaxAcc;
+  // Accumulator barriers, one pair per epilogue group and not per accumulator: tile i's are
+  // those of group i % 4 whatever n_acc.  (Two groups that share an accumulator would each see every
+  // second phase of one barrier, and a phase's parity does not tell it from the one two later.)
+  uint64_t* tfull_bar = empty_bar + STAGES;        // [kSGroups]
+  uint64_t* tempty_bar = tfull_bar + kSGroups;     // [kSGroups]
+  uint64_t* qfull_bar = tempty_bar + kSGroups;
   uint64_t* qempty_bar = qfull_bar + 2;
   uint64_t* drain_bar = qempty_bar + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain_bar + 1);
@@ -149,9 +152,9 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
       mbar_init(&full_bar[s], 1);
       mbar_init(&empty_bar[s], 1);
     }
-    for (int a = 0; a < kMaxAcc; ++a) {
-      mbar_init(&tfull_bar[a], 1);
-      mbar_init(&tempty_bar[a], 4);
+    for (int g = 0; g < kSGroups; ++g) {
+      mbar_init(&tfull_bar[g], 1);
+      mbar_init(&tempty_bar[g], 4);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&qfull_bar[i], 1);
@@ -259,7 +262,9 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
       const int qs = (qcount - 1) % NQB;
       const int s = i % STAGES;
       const int acc = i % n_acc;
-      if (i >= n_acc && !mbar_wait_warp(&tempty_bar[acc], ((i / n_acc) & 1) ^ 1, p.status, abort_flag)) break;
+      // the accumulator's tile before this one has been read
+      const int prev = i - n_acc;
+      if (prev >= 0 && !mbar_wait_warp(&tempty_bar[prev % kSGroups], (prev / kSGroups) & 1, p.status, abort_flag)) break;
       const uint32_t a_lo = desc_k(smem_u32(kstage + s * KTILE));
       const uint32_t b_lo = desc_k(smem_u32(qbuf + qs * qbytes));
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * p.acc_stride);
@@ -270,14 +275,14 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
         tc_mma_ss(lead, d_tmem, a_lo + ((ks >> 2) * KHALF + (ks & 3) * 32) / 16,
                   b_lo + ((ks >> 2) * b_half + (ks & 3) * 32) / 16, idesc, ks > 0 ? 1u : 0u);
       tc_commit(lead, &empty_bar[s]);
-      tc_commit(lead, &tfull_bar[acc]);
+      tc_commit(lead, &tfull_bar[i % kSGroups]);
       if (unit_ends) tc_commit(lead, &qempty_bar[qs]);
     }
     // every MMA this warp issued has completed before TMEM is released
     tc_commit(lead, drain_bar);
     mbar_wait(drain_bar, 0, p.status, nullptr);
   } else {
-    // ---------------------------------------------------------------- epilogue (2 groups of 4 warps)
+    // ---------------------------------------------------------------- epilogue (kSGroups groups of 4 warps)
     if (!RAGGED && n > 0 && warp == 2)           // the first unit's window LSE into L2 meanwhile
       prefetch_lines_l2(p.lse_win + (size_t)unit_first * p.nq_rows, (size_t)p.nq_rows * 4, lane, 32);
     grid_dependency_wait();                      // the window LSE is carried from earlier kernels
@@ -290,7 +295,7 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
     int win0 = p.t_ctx - p.window;              // position of window row 0 (of the current unit)
     int mid_end = p.mid_end;                    // end of the current unit's middle
     int cur_unit = -1, unit = unit_first;
-    for (int i = grp; i < n; i += 4) {
+    for (int i = grp; i < n; i += kSGroups) {
       int tt;
       locate(first + i, unit, tt);
       if (unit != cur_unit) {
@@ -310,7 +315,7 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
         cur_unit = unit;
       }
       const int acc = i % n_acc;
-      if (!mbar_wait(&tfull_bar[acc], (i / n_acc) & 1, p.status, abort_flag)) break;
+      if (!mbar_wait(&tfull_bar[grp], (i / kSGroups) & 1, p.status, abort_flag)) break;
       tc_fence_after();
       const int key_tile0 = p.n_sink + kSKeys * tt;
       const int key = key_tile0 + quad * 32 + lane;
@@ -357,7 +362,7 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty_bar[acc]);
+      if (lane == 0) mbar_arrive(&tempty_bar[grp]);
       if (key < mid_end) p.score[(size_t)unit * p.n_mid_pad + (key - p.n_sink)] = (sum0 + sum1) + (sum2 + sum3);
     }
   }
