@@ -5,7 +5,8 @@
 // each CTA derives the same threshold by itself.  What bounds it is the chain of exchanges
 // (four cluster barriers) and the slowest CTA's passes over its own items.  A select call over
 // 8 units of 128K positions: 377 us with one CTA per unit (scores re-read by every radix pass),
-// 70 us here (score kernel 51 us); 2 units of 200K: 482 -> 53 us.
+// 65.3 us here with whole histograms crossing the cluster and the scores loaded row by row, 54.8 with
+// two-level histograms and every load in flight at once (score kernel 45 us of it).
 //
 // The kept set is the k items of largest (value, lowest index): as 64-bit keys
 // (value bits, ~index) they are distinct, so the threshold is one key and an item is kept
@@ -22,6 +23,8 @@ namespace cg = cooperative_groups;
 namespace bd {
 
 constexpr int kTMaxCluster = 8;     // CTAs per unit: the portable cluster size
+constexpr int kTGroups = 64;        // groups of kTFine adjacent histogram bins
+constexpr int kTFine = kBins / kTGroups;
 
 struct TopkLongSmem {
   uint32_t bins[kBins];             // own histogram, then all ranks' boundary-bin items
@@ -29,11 +32,13 @@ struct TopkLongSmem {
   uint32_t digit[2][256];           // radix passes (crowded boundary bin)
   uint32_t wsum[32];
   float2 range[kTMaxCluster];       // every rank's (min, max)
+  uint32_t group[kTMaxCluster][kTGroups];    // every rank's items per group of bins
+  uint32_t fine[kTFine][kTMaxCluster];       // the boundary group's bins, every rank's
   uint32_t chosen[kTMaxCluster];    // every rank's kept positions
   uint32_t in_bin[kTMaxCluster];    // every rank's boundary-bin items
   float wmin[32], wmax[32];
   uint64_t key;
-  uint32_t total, bin, above, count, n_cand;
+  uint32_t total, bin, above, count, n_cand, group_star, group_above;
   int first_kept;
 };
 static_assert(sizeof(uint32_t) * kBins >= sizeof(uint64_t) * kBinCandMax, "all ranks' items fit the bins");
@@ -112,14 +117,23 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_cluster_kernel(const Top
     }
     return v > 0.f ? __float_as_uint(v) : 0u;
   };
-  const int w_item0 = item0 + warp * rows * 32;
+  const int w_item0 = item0 + warp * rows * 32, w_end = min(n, w_item0 + 32 * rows);   // the warp's items
+  constexpr uint32_t kNoItem = ~0u;               // past the items (a score's bits are never this)
   uint32_t u[ROWS > 0 ? ROWS : 1];
-  if (ROWS > 0) {
+  if (ROWS > 0 && CHUNK) {
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
       const int i = w_item0 + 32 * r + lane;
-      u[r] = r < rows && i < n ? value(i) : 0u;
+      u[r] = i < w_end ? value(i) : kNoItem;
     }
+  } else if (ROWS > 0) {                          // all loads in flight before the first is used
+    const float* base = sc + w_item0 + lane;
+    const int left = w_end - w_item0 - lane;
+    float x[ROWS > 0 ? ROWS : 1];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) x[r] = 32 * r < left ? __ldcg(base + 32 * r) : 0.f;
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) u[r] = 32 * r < left ? (x[r] > 0.f ? __float_as_uint(x[r]) : 0u) : kNoItem;
   }
   // f(r, i, bits) for every item of this thread, in item order
   auto each = [&](auto f) {
@@ -127,7 +141,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_cluster_kernel(const Top
 #pragma unroll
       for (int r = 0; r < ROWS; ++r) {
         const int i = w_item0 + 32 * r + lane;
-        if (r < rows && i < n) f(r, i, u[r]);
+        if (u[r] != kNoItem) f(r, i, u[r]);
       }
     } else {
 #pragma unroll 4
@@ -183,37 +197,69 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_cluster_kernel(const Top
       return min(kBins - 1, max(0, (int)((__uint_as_float(bits) - vmin) * scale)));
     };
     each([&](int, int, uint32_t bits) { atomicAdd(&S.bins[bin_of(bits)], 1u); });
-    cluster.sync();
-    constexpr int BPT = kBins / kTopkThreads;
-    static_assert(BPT == 4, "a thread's bins are one 16-byte vector");
-    uint32_t hb[BPT] = {0, 0, 0, 0};
+    __syncthreads();
+    // The boundary bin in two levels, so that little crosses the cluster: sums of 64 bins go to every
+    // rank, then each reads the 64 bins of the group that holds the k-th item (every rank
+    // reading every histogram whole, 1 MB per cluster, took 4.6 us against 1.5).
+    static_assert(kBins == 4 * kTopkThreads && kTFine == 64 && kTGroups == 64, "16 threads sum a group of bins");
+    {
+      const uint4 h = reinterpret_cast<const uint4*>(S.bins)[tid];
+      uint32_t sum = (h.x + h.y) + (h.z + h.w);
 #pragma unroll
-    for (int q = 0; q < kTMaxCluster; ++q) {
-      if (q < C) {
-        const uint4 h = reinterpret_cast<const uint4*>(cluster.map_shared_rank(S.bins, q))[tid];
-        hb[0] += h.x;
-        hb[1] += h.y;
-        hb[2] += h.z;
-        hb[3] += h.w;
-      }
+      for (int off = 8; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+      if ((lane & 15) < C) *cluster.map_shared_rank(&S.group[rank][tid >> 4], lane & 15) = sum;
     }
-    const uint32_t incl = block_inclusive(hb[0] + hb[1] + hb[2] + hb[3], S.wsum, &S.total);
-    uint32_t above = (uint32_t)n - incl;          // items in the bins above this thread's
+    cluster.sync();
+    // the entry of 64 (two per lane of warp 0) that holds the k-th item, `over` items being in
+    // later entries than these 64: its index, items after it, its own
+    auto find = [&](uint32_t h0, uint32_t h1, uint32_t in_all, uint32_t over, auto found) {
+      uint32_t incl = h0 + h1;
 #pragma unroll
-    for (int j = BPT - 1; j >= 0; --j) {
-      if (above < (uint32_t)k && (uint32_t)k <= above + hb[j]) {
-        S.bin = (uint32_t)(tid * BPT + j);
-        S.above = above;
-        S.count = hb[j];
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
       }
-      above += hb[j];
+      const uint32_t after1 = over + in_all - incl, after0 = after1 + h1;
+      if (after1 < (uint32_t)k && (uint32_t)k <= after1 + h1) found(2 * lane + 1, after1, h1);
+      if (after0 < (uint32_t)k && (uint32_t)k <= after0 + h0) found(2 * lane, after0, h0);
+    };
+    if (warp == 0) {
+      uint32_t h0 = 0, h1 = 0;
+      for (int q = 0; q < C; ++q) {
+        h0 += S.group[q][2 * lane];
+        h1 += S.group[q][2 * lane + 1];
+      }
+      find(h0, h1, (uint32_t)n, 0u, [&](int g, uint32_t after, uint32_t own) {
+        S.group_star = (uint32_t)g;
+        S.group_above = after;
+        S.total = own;
+      });
+    }
+    __syncthreads();
+    if (tid < kTFine * kTMaxCluster) {
+      const int q = tid % kTMaxCluster, j = tid / kTMaxCluster;
+      S.fine[j][q] = q < C ? cluster.map_shared_rank(S.bins, q)[S.group_star * kTFine + j] : 0u;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      uint32_t h0 = 0, h1 = 0;
+#pragma unroll
+      for (int q = 0; q < kTMaxCluster; ++q) {
+        h0 += S.fine[2 * lane][q];
+        h1 += S.fine[2 * lane + 1][q];
+      }
+      find(h0, h1, S.total, S.group_above, [&](int j, uint32_t after, uint32_t own) {
+        S.bin = S.group_star * kTFine + (uint32_t)j;
+        S.above = after;
+        S.count = own;
+      });
     }
     __syncthreads();
     const int bstar = (int)S.bin;
     const uint32_t nc = S.count;
     if (nc <= (uint32_t)kBinCandMax) {
       // ---- the bin's items of every rank, ranked exactly
-      if (tid < C) S.in_bin[tid] = cluster.map_shared_rank(S.bins, tid)[bstar];
+      if (tid < C) S.in_bin[tid] = S.fine[bstar % kTFine][tid];
       each([&](int, int i, uint32_t bits) {
         if (bin_of(bits) == bstar) S.cand[atomicAdd(&S.n_cand, 1u)] = key_of(i, bits);
       });
@@ -277,7 +323,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) topk_cluster_kernel(const Top
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
       const int i = w_item0 + 32 * r + lane;
-      masks[r] = __ballot_sync(0xffffffffu, any && r < rows && i < n && key_of(i, u[r]) >= threshold);
+      masks[r] = __ballot_sync(0xffffffffu, any && u[r] != kNoItem && key_of(i, u[r]) >= threshold);
       cnt += __popc(masks[r]);
     }
   } else {
