@@ -18,6 +18,7 @@
 //   warps 0..3  consumers on mma.sync (bd_attn_warp.cuh): the GQA group's packed query
 //               rows are the N side of S^T = K Q^T.
 #include <algorithm>
+#include <climits>
 
 #include "bd_attn_warp.cuh"
 #include "bd_common.cuh"
@@ -30,12 +31,12 @@ constexpr int kVKeys = 64;            // keys per pipeline stage
 constexpr int kVConsumers = 4;        // consumer warps
 constexpr int kVThreads = 160;        // + one producer warp
 constexpr int kVStages = 5;
-// Query rows of a KV head that verify_kernel takes: three n8 tiles, up to which it streams at
+// Most query rows of a KV head that verify_kernel takes: three n8 tiles, up to which it streams at
 // memory speed and starts sooner; with more, every tile of keys costs another pass of mma.sync
-// and verify_tc_kernel is faster.  64 units of 16K, both sides measured: 24 rows 86.4 us here, 87.3
-// there; 28 rows 154.5 / 85.4; 84 rows 313.8 / 89.1.  8 units of 4K: 24 rows 10.5 / 11.2, 36 rows
-// 13.4 / 12.6, 84 rows 19.2 / 13.4.
+// and verify_tc_kernel is faster.  64 units of 16K, both sides measured: 28 rows 154.5 us here, 85.4
+// there; 84 rows 313.8 / 89.1.  8 units of 4K: 24 rows 10.5 / 11.2, 36 rows 13.4 / 12.6, 84 rows 19.2 / 13.4.
 constexpr int kVMaxRows = 24;
+constexpr int kVTcRows = 16;          // query rows from which a large batch moves already
 constexpr int kVTcMaxRows = 256;      // query rows of one unit of verify_tc_kernel: two M tiles
 constexpr int kVMaxChunks = 3;        // row chunks of one (sequence, KV head): 768 query rows in all
 
@@ -378,15 +379,26 @@ int occupancy(const KernelInfo& k) {
 
 }  // namespace
 
+// Blocks that verify_kernel could take but verify_tc_kernel streams faster: a third n8 tile slows
+// every tile of keys in the one (8 rows 81.5 us, 24 rows 86.3 us for 64 units of 16K), while the other
+// costs the same up to 128 rows and wants a merge launch, which pays once the batch fills the SMs by itself.
+// verify_kernel / verify_tc_kernel, d 128, us: 64 units, 24 rows, of 1K 17.0 / 16.3, 4K 31.9 / 30.2, 16K 87.1 / 85.7;
+// 128 units, 21 rows, of 4K 51.4 / 49.0; 12 rows: 15.0 / 16.3, 29.8 / 29.9, 85.3 / 85.3; 32 units, 24 rows, of 16K 47.9 /
+// 49.4; d 64, 64 units of 16K 49.8 / 58.5; per-sequence lengths, 21 rows 48.2 / 48.4.
+static bool tc_streams_better(const bd_shape& s, int n_q) {
+  return s.head_dim == 128 && s.seq_lens == nullptr && 3L * s.batch * s.h_kv > current_sm_count() &&
+         (long)s.t_ctx + n_q >= 1024;
+}
+
 bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   const int group = s.h_q / s.h_kv;
   const long rows_total = (long)group * n_q;
-  const bool tc = rows_total > kVMaxRows;
+  const bool ragged = s.seq_lens != nullptr;
+  const bool tc = rows_total > kVMaxRows || (rows_total > kVTcRows && tc_streams_better(s, n_q));
   // more query rows than one CTA holds: chunks of equal size
   const int chunks = tc ? (int)((rows_total + kVTcMaxRows - 1) / kVTcMaxRows) : 1;
   if (chunks > kVMaxChunks) return false;
   const int nq_rows = (int)((rows_total + chunks - 1) / chunks);
-  const bool ragged = s.seq_lens != nullptr;
   const int nt = nq_rows <= 8 ? 1 : 3;
   const int q_tiles = tc ? (nq_rows > 128 ? 2 : 1) : 0;
   KernelInfo k = {nullptr, 0, 0};
@@ -452,10 +464,12 @@ size_t verify_partials_bytes(const bd_shape& s, const VerifyPlan& plan) {
 }
 
 size_t verify_region_bytes(const bd_shape& s, int n_q) {
-  VerifyPlan vp;
-  size_t bytes = verify_plan(s, n_q, &vp) ? verify_partials_bytes(s, vp) : 0;
-  const int fewer = kVMaxRows / (s.h_q / s.h_kv);
-  if (fewer >= 1 && fewer < n_q && verify_plan(s, fewer, &vp)) bytes = std::max(bytes, verify_partials_bytes(s, vp));
+  size_t bytes = 0;
+  for (const int rows : {INT_MAX, kVMaxRows, kVTcRows}) {
+    const int n = std::min(n_q, rows / (s.h_q / s.h_kv));
+    VerifyPlan vp;
+    if (n >= 1 && verify_plan(s, n, &vp)) bytes = std::max(bytes, verify_partials_bytes(s, vp));
+  }
   return bytes;
 }
 

@@ -69,3 +69,9 @@ def test_growing_scores(n_q):
 
 def test_many_units_per_cta():
     block(24, 64, 16, 64, 150, 8)
+
+
+@pytest.mark.parametrize("rows", [16, 17, 24])
+def test_few_rows_of_a_large_batch(rows):
+    block(16, 8, 4, 128, 1100, rows // 2 if rows % 2 == 0 else 9, repeat=1)
+    block(60, rows, 1, 128, 1100, 1, repeat=1)
