@@ -212,7 +212,8 @@ class Step:
             sel = 1
         else:
             sel = 2 + (1 if self.sel_mode == "self" else 0)
-        return self.wl.layers * (sel + self.wl.gamma + 1)
+        # the verify block: its kernel and the merge of its segments
+        return self.wl.layers * (sel + self.wl.gamma + 2)
 
     def run(self, marks=None, select=True):
         """One step; marks = [select, draft, verify, end] timing events (or None).  With
@@ -361,7 +362,7 @@ def gpu_arm(args):
         "algorithmic_bytes_per_step": layer_bytes,
         "breakdown_us": {k: round(v, 2) for k, v in phase_us.items()},
         "roofline": {
-            "kernel": "verify_kernel (bd_verify_attn)",
+            "kernel": "verify_tc_kernel and its merge (bd_verify_attn)",
             "bound": "hbm",
             "achieved": round(achieved, 1),
             "peak": peak,
@@ -369,8 +370,8 @@ def gpu_arm(args):
             "unit": "GB/s",
             "frac": round(achieved / peak, 3),
             "bytes_per_launch": verify_launch_bytes,
-            "traffic": profiled_traffic("verify_kernel", wl.name, ("bd_verify.cu", "bd_attn_warp.cuh", "bd_common.cuh")),
-            "traffic_source": "profiles/verify_kernel_%s.md (ncu dram__bytes_read.sum + dram__bytes_write.sum)" % wl.name,
+            "traffic": profiled_traffic("verify_tc_kernel", wl.name, ("bd_verify_tc.cu", "bd_verify.cuh", "bd_common.cuh")),
+            "traffic_source": "profiles/verify_tc_kernel_%s.md (ncu dram__bytes_read.sum + dram__bytes_write.sum)" % wl.name,
         },
         "gpu_launches": step.launches_per_step() * args.steps,
         "clocks": clocks,
@@ -435,7 +436,7 @@ def extras(step, args):
     us = time_per_step(lambda: step.run(select=False), n, gs)
     b = (per["draft"] + per["verify"]) * wl.layers
     out["amortized_step"] = {"us_per_step": round(us, 2), "GB/s": round(b / (us * 1e-6) / 1e9, 1),
-                             "bytes_per_step": b, "launches_per_step": wl.layers * (wl.gamma + 1)}
+                             "bytes_per_step": b, "launches_per_step": wl.layers * (wl.gamma + 2)}
 
     # greedy acceptance (Eq. accept, Algorithm 2): arg max of every drafter pass and of the
     # verify block over a Llama-3 vocabulary, then the prefix test; synthetic bf16 logits
