@@ -1496,7 +1496,7 @@ bool lse_plan(const bd_shape& s, int window, LsePlan* plan) {
     max_seg = kLMaxSeg;
   } else {
     grid = (int)((total + tpc - 1) / tpc);
-    for (long u = 0; u < units; ++u)
+    for (long u = 0; u < std::min<long>(units, tpc); ++u)   // (the offsets repeat after tpc units)
       max_seg = std::max(max_seg, (int)((u * tpu + tpu - 1) / tpc - (u * tpu) / tpc + 1));
   }
   plan->nq_rows = (int)rows;

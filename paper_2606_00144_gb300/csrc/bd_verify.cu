@@ -434,7 +434,7 @@ bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   plan->tiles_per_cta = (int)vtpc;
   plan->grid = (int)((vtotal + vtpc - 1) / vtpc);
   int max_seg = 1;
-  for (long u = 0; u < units; ++u) {
+  for (long u = 0; u < std::min(units, vtpc); ++u) {   // (units' offsets in the CTA ranges repeat after vtpc units)
     const int c0 = tile_owner((int)(u * tpu), tpu, a, (int)vtpc);
     const int c1 = tile_owner((int)(u * tpu + tpu - 1), tpu, a, (int)vtpc);
     max_seg = std::max(max_seg, c1 - c0 + 1);
