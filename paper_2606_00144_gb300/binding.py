@@ -124,11 +124,17 @@ def bd_workspace_size(shape: BdShape, op: int, budget: int, n_q: int) -> int:
 
 
 class Workspace:
-    """A zero-filled device buffer sized for a set of operations (see bd_workspace_size)."""
+    """A device buffer sized for a set of operations (see bd_workspace_size), zero-filled: as a
+    whole, or with ``units`` (batch * h_kv) given only the status word and the arrival counters, the
+    part that the kernels read before they write it."""
 
-    def __init__(self, nbytes: int, device=None):
+    def __init__(self, nbytes: int, device=None, units: int | None = None):
         self.nbytes = int(max(nbytes, 512))
-        self.buf = torch.zeros(self.nbytes, dtype=torch.uint8, device=device or "cuda")
+        if units is None:
+            self.buf = torch.zeros(self.nbytes, dtype=torch.uint8, device=device or "cuda")
+        else:
+            self.buf = torch.empty(self.nbytes, dtype=torch.uint8, device=device or "cuda")
+            self.buf[:256 + -(-4 * units // 256) * 256].zero_()
 
     @classmethod
     def for_step(cls, shape: BdShape, budget: int, window: int, gamma: int, device=None):

@@ -90,6 +90,9 @@ class SpecStep:
         if out is None:
             out = torch.empty(self.shape.batch, self.shape.h_q, self.window, dtype=torch.float32,
                               device=k_cache.device)
-        ws = B.Workspace(B.bd_workspace_size(sh, B.BD_OP_VERIFY, 1, self.window), k_cache.device)
+        # (a workspace of this call's own; its size covers a block with an output too, 17 MB for 64
+        # units of 16K, so only the words that have to be zero are filled)
+        ws = B.Workspace(B.bd_workspace_size(sh, B.BD_OP_VERIFY, 1, self.window), k_cache.device,
+                         units=sh.batch * sh.h_kv)
         B.bd_verify_attn(sh, q_win, self.window, k_cache, None, None, out, ws, stream)
         return out
