@@ -373,25 +373,30 @@ static int draft_pos_slots(const DraftPlan& plan) {
 // tile up to 8, two beyond).
 int draft_group_instance(int g) { return g <= 1 ? 1 : g <= 2 ? 2 : g <= 4 ? 4 : g <= 8 ? 8 : 16; }
 
-// Clusters of c CTAs of a LONG instance (one CTA per SM) that the device holds at once.
-static long long_clusters(int d, int g_kernel, int c) {
+// Clusters of c CTAs that the device holds at once: LONG instances at one CTA per SM, short ones
+// with two tile buffers at two.  (A GPC's SMs are shared out by whole clusters, so it is fewer than the SMs' CTAs
+// divided by c.)
+static long clusters_held(int d, int g_kernel, bool longs, int c) {
   static thread_local int cache_dev = -1;
-  static thread_local int cache[kDMaxCluster + 1];
+  static thread_local int cache[2][kDMaxCluster + 1];
   int dev = 0;
+  const int per_sm = longs ? 1 : 2;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     (void)cudaGetLastError();
-    return current_sm_count() / c;
+    return per_sm * current_sm_count() / c;
   }
   if (dev != cache_dev) {
-    for (int& n : cache) n = -1;
+    for (auto& row : cache)
+      for (int& n : row) n = -1;
     cache_dev = dev;
   }
-  if (cache[c] < 0) {
-    void* fn = pick(d, g_kernel, true);
-    const size_t smem = 200 * 1024;
+  int& held = cache[longs][c];
+  if (held < 0) {
+    void* fn = pick(d, g_kernel, longs);
+    const size_t smem = (longs ? 200 : 100) * 1024;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c);
-    cfg.blockDim = dim3(2 * kDLongRows);
+    cfg.blockDim = dim3(2 * (longs ? kDLongRows : kDRows));
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
@@ -403,11 +408,11 @@ static long long_clusters(int d, int g_kernel, int c) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
-      n = current_sm_count() / c;
+      n = per_sm * current_sm_count() / c;
     }
-    cache[c] = n;
+    held = n;
   }
-  return cache[c];
+  return held;
 }
 
 // One cluster per unit merges in shared memory; several leave a partial each.
@@ -427,16 +432,19 @@ bool draft_plan(const bd_shape& s, int budget, int n_steps, size_t room, DraftPl
   const int g = s.h_q / s.h_kv;
   if (g < 1 || g > 16 || !pick(s.head_dim, draft_group_instance(g), false)) return false;
   const long entries = (long)budget + n_steps;
+  const int g_kernel = draft_group_instance(g);
   // one tile per CTA up to a cluster of 8, but no more CTAs than one wave holds at the
   // occupancy the slice's stage count gives (three single-stage or two double-buffered
-  // CTAs per SM, draft_stages): a second wave would repeat the pass's whole latency chain
+  // CTAs per SM, draft_stages): a second wave would repeat the pass's whole latency chain.  With
+  // two buffers counted in whole clusters: 48 units of 2K rows took 16.5 us a pass in clusters of six, some
+  // of which waited for a second wave, 11.4 in clusters of five; 40 units of 2K 14.5 / 9.9.
   const long units = (long)s.batch * s.h_kv;
   const long sms = current_sm_count();
   int n_split = (int)std::min<long>((entries + kDRows - 1) / kDRows, kDMaxCluster);
   for (; n_split > 1; --n_split) {
     const long rps = (entries + n_split - 1) / n_split, ctas = units * n_split;
     const bool dbuf = (rps > kDRows && ctas <= 2 * sms) || rps > 2 * kDRows;
-    if (ctas <= (dbuf ? 2 : 3) * sms) break;
+    if (ctas <= (dbuf ? 2 : 3) * sms && (!dbuf || units <= clusters_held(s.head_dim, g_kernel, false, n_split))) break;
   }
   n_split = std::max(n_split, 1);
   const long rows_per_split = (entries + n_split - 1) / n_split;
@@ -446,7 +454,6 @@ bool draft_plan(const bd_shape& s, int budget, int n_steps, size_t room, DraftPl
   plan->n_clusters = 1;
   plan->longs = false;
   // the row table of a CTA's slice sits in shared memory beside its tiles
-  const int g_kernel = draft_group_instance(g);
   // A LONG instance where its estimate is the shorter: a fixed cost, one per tile a CTA walks
   // (both fitted to passes of 4 units of 1K to 8K rows), one where clusters meet in memory.  Per pass,
   // d 128, short / LONG measured: 4 units of 1K rows 5.1 / 4.8 us, 2K 7.2 / 5.8, 8K 16.2 / 7.7; 8 units of
@@ -454,7 +461,7 @@ bool draft_plan(const bd_shape& s, int budget, int n_steps, size_t room, DraftPl
   // L2's rate; stays short).  Clusters of two CTAs gained nothing.
   double best_us = 3.1 + 1.0 * ((rows_per_split + kDRows - 1) / kDRows);
   for (int c = kDMaxCluster; c >= 3; --c) {
-    const long cap = long_clusters(s.head_dim, g_kernel, c);
+    const long cap = clusters_held(s.head_dim, g_kernel, true, c);
     for (int k = 1; k <= kDMaxParts && units * k <= cap; ++k) {
       const long rps = (entries + c * k - 1) / (c * k);
       const double us = 3.0 + 1.33 * ((rps + kDLongRows - 1) / kDLongRows) + (k > 1 ? 2.05 : 0.0);
