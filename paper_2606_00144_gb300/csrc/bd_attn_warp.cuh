@@ -12,6 +12,8 @@
 // K/V sub-tiles are read from shared memory in the TMA SWIZZLE_128B layout (sw128_offset).
 #pragma once
 
+#include <climits>
+
 #include "bd_common.cuh"
 
 namespace bd {
@@ -61,12 +63,14 @@ struct WarpAttn {
 
   // One 16-key sub-tile at rows kb..kb+15 of the K (and V) tile.  ok(key_offset, nt, e)
   // says whether key kb + key_offset (key_offset = gid or gid + 8) is visible to query
-  // column 8*nt + 2*tig + e of this warp.
+  // column 8*nt + 2*tig + e of this warp.  V rows past v_last of the tile may hold anything (a
+  // weight of 0 times NaN would be NaN): row v_last is read in their place.
   template <typename Visible>
   __device__ __forceinline__ void step(uint32_t kbase, uint32_t vbase, uint32_t half_bytes, int kb,
                                        const uint32_t (&bq)[NT][KS][2], float scale_log2, int lane,
-                                       Visible ok) {
+                                       Visible ok, int v_last = INT_MAX) {
     const int gid = lane >> 2;
+    const int v_row = min(kb + (lane & 7) + 8 * (lane >> 4), v_last);
     float s[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
@@ -128,8 +132,7 @@ struct WarpAttn {
 #pragma unroll
     for (int mt = 0; mt < KS; ++mt) {
       uint32_t a[4];
-      ldmatrix_x4_trans(a, vbase + sw128_offset(kb + (lane & 7) + 8 * (lane >> 4), 16 * mt + 8 * ((lane >> 3) & 1),
-                                                half_bytes));
+      ldmatrix_x4_trans(a, vbase + sw128_offset(v_row, 16 * mt + 8 * ((lane >> 3) & 1), half_bytes));
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
         mma_16816(o[mt][nt], a, bp[nt][0], bp[nt][1]);

@@ -202,8 +202,11 @@ __global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
       for (int sub = 0; sub < SUBS; ++sub) {
         const int kb = 16 * (warp + kVConsumers * sub);
         const int key_base = tile * kVKeys + kb;
+        // (a shorter sequence's last tile reaches cache rows past its own block, which nobody has promised to
+        // be finite; past the longest block the tensor map reads zeros)
         wa.step(kbase, vbase, HALF_BYTES, kb, bq, p.scale_log2, lane,
-                [&](int ko, int nt, int e) { return key_base + ko <= lim[nt][e]; });
+                [&](int ko, int nt, int e) { return key_base + ko <= lim[nt][e]; },
+                UNIFORM ? INT_MAX : t_unit + p.n_q - 1 - tile * kVKeys);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty_bar[s]);

@@ -43,6 +43,21 @@ struct VerifyTcSmem {
   static constexpr size_t kTotal = kTFixed + (size_t)(NQT + SLOTS) * TILE;
 };
 
+// Rows [r0, 128) of a V tile in shared memory become zero, by one warp, before that warp's MMAs read them.
+// With per-sequence lengths the last tile of a sequence shorter than the longest one reaches cache rows
+// past its own block, which nobody has promised to be finite, and a weight of 0 times NaN is NaN.
+template <int D>
+__device__ __forceinline__ void clear_rows(uint8_t* tile, int r0, int lane) {
+  if (r0 >= kVTcKeys) return;
+  constexpr int CH = D / 8, PER = 32 / CH;          // 16-byte chunks of a row; rows at a time
+  const int c = lane % CH;
+  uint8_t* at = tile + c / 8 * kTHalf + c % 8 * 16;
+#pragma unroll 1
+  for (int r = r0 + lane / CH; r < kVTcKeys; r += PER) *reinterpret_cast<uint4*>(at + r * 128) = make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy_async_smem();
+  __syncwarp();
+}
+
 // UNIFORM: one shared context length; the other instance lays out per-sequence lengths.
 template <int D, int NQT, bool UNIFORM>
 __global__ void __launch_bounds__(kVTcThreads, 1) verify_tc_kernel(const VerifyParams p,
@@ -65,6 +80,7 @@ __global__ void __launch_bounds__(kVTcThreads, 1) verify_tc_kernel(const VerifyP
   uint64_t* drain_bar = o_free + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  int* live_s = reinterpret_cast<int*>(tmem_slot + 2);      // [SLOTS] per-sequence lengths: the block's rows in a segment's last V tile
   float2* ml_s = reinterpret_cast<float2*>(smem + 1024);    // [2][128] (m, l) of the two groups
   uint8_t* qbuf = smem + 1024 + 2 * 128 * sizeof(float2);   // NQT x TILE
   uint8_t* ring = qbuf + NQT * TILE;                        // SLOTS x TILE
@@ -143,6 +159,7 @@ __global__ void __launch_bounds__(kVTcThreads, 1) verify_tc_kernel(const VerifyP
         const int tb = map.first_tile(unit, v0), te = map.end_tile(unit, v1), n = te - tb;
         if (n <= 0) continue;
         const int kv_unit = unit / p.row_chunks;
+        const int t_unit = UNIFORM ? 0 : p.seq_lens[kv_unit / p.h_kv];   // (on its way; used at the segment's end)
         // entry i of the segment: K of tile 0 or (odd i) of tile (i + 1) / 2, else V
         auto entry_tile = [&](int i) { return i == 0 ? 0 : i == 2 * n - 1 ? n - 1 : (i & 1) ? (i + 1) >> 1 : (i >> 1) - 1; };
         auto issue = [&](int i) {
@@ -155,6 +172,7 @@ __global__ void __launch_bounds__(kVTcThreads, 1) verify_tc_kernel(const VerifyP
             waited = true;
           }
           const CUtensorMap* m = i == 0 || ((i & 1) && i != 2 * n - 1) ? &kmap : &vmap;
+          if (!UNIFORM && i == 2 * n - 1) live_s[s] = min(max(t_unit, 1), p.t_ctx) + p.n_q - key0;
           mbar_arrive_expect_tx(&full_bar[s], TILE);
 #pragma unroll
           for (int h = 0; h < D / 64; ++h) tma_load_3d(ring + s * TILE + h * kTHalf, m, &full_bar[s], 64 * h, key0, kv_unit);
@@ -217,6 +235,7 @@ __global__ void __launch_bounds__(kVTcThreads, 1) verify_tc_kernel(const VerifyP
           const int r = base + v_pos(i, n), s = r % SLOTS;
           if (j == 1 && seg > 0) ok = mbar_wait_warp(o_free, (seg - 1) & 1, p.status, abort_flag);
           if (ok && qt == 0) ok = mbar_wait_warp(&full_bar[s], (r / SLOTS) & 1, p.status, abort_flag);
+          if (!UNIFORM && ok && i == n - 1 && qt == 0) clear_rows<D>(ring + s * TILE, live_s[s], lane);
           if (ok) ok = mbar_wait_warp(&p_ready[b], (jj >> 1) & 1, p.status, abort_flag);
           if (!ok) break;
           tc_fence_after();
