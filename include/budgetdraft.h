@@ -133,7 +133,8 @@ enum {
  *               chunk == s > 1: the top floor((budget - n_sink - n_recent)/s) chunks,
  *                 chunk c = positions [c s, c s + s) within the middle, scored by the
  *                 sum of its members;
- *          ties go to the lower position (chunk).  If budget >= t_ctx, keep = [0, t_ctx).
+ *          ties go to the lower position (chunk); a score that is NaN counts as 0.
+ *          If budget >= t_ctx, keep = [0, t_ctx).
  *
  *   k_cache     bf16 [batch, h_kv, t_cap, d]; rows [0, t_ctx) are read.
  *   q_window    bf16 [batch, h_q, window, d]: queries of positions t_ctx-W .. t_ctx-1.

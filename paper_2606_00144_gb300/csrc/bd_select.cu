@@ -363,7 +363,11 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty_bar[grp]);
-      if (key < mid_end) p.score[(size_t)unit * p.n_mid_pad + (key - p.n_sink)] = (sum0 + sum1) + (sum2 + sum3);
+      // (a NaN, from one in a key, a query or a normaliser, counts as 0: ranked by its bits it would be above
+      // every threshold while the histogram has it in the lowest bin, and more items than the budget holds
+      // would be written)
+      if (key < mid_end)
+        p.score[(size_t)unit * p.n_mid_pad + (key - p.n_sink)] = fmaxf((sum0 + sum1) + (sum2 + sum3), 0.f);
     }
   }
 
