@@ -103,7 +103,8 @@ enum { BD_OP_SELECT = 1, BD_OP_DRAFT = 2, BD_OP_VERIFY = 3 };
  * Workspace bytes needed by one operation on `shape` (0 on invalid input).
  *   BD_OP_SELECT: budget = B, n_q = window W (window queries per head);
  *   BD_OP_DRAFT:  budget = B, n_q = the largest step_j + 1 that will be passed;
- *   BD_OP_VERIFY: budget ignored, n_q = queries per head in the block.
+ *   BD_OP_VERIFY: budget ignored, n_q = queries per head in the block, or the most that
+ *                 will be passed (with or without an output).
  * The size depends on the current device's SM count.  Sizes for different ops may
  * be satisfied by one buffer of the largest of them.
  */

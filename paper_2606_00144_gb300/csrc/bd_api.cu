@@ -127,14 +127,6 @@ void* region(void* ws, int units) { return static_cast<uint8_t*>(ws) + ws_region
 
 bool group_supported_by_draft(int g) { return g >= 1 && g <= 16; }
 
-// bd_verify_attn without an output: the block's rows are the last n_q positions of a context
-// of t_ctx + n_q
-bd_shape block_context(const bd_shape& s, int n_q) {
-  bd_shape ls = s;
-  ls.t_ctx = s.t_ctx + n_q;
-  return ls;
-}
-
 }  // namespace
 
 #define BD_TRY(x)                  \
@@ -169,7 +161,7 @@ size_t bd_workspace_size(const bd_shape* shape, int op, int budget, int n_q) {
       const size_t base = ws_region_offset(units);
       const size_t a = verify_plan(s, n_q, &vp) ? base + verify_region_bytes(s, n_q) : 0;
       const size_t b = (long long)s.t_ctx + n_q <= s.t_cap && lse_plan(block_context(s, n_q), n_q, &lp)
-                           ? base + lp.part_bytes
+                           ? base + lse_region_bytes(s, n_q)
                            : 0;
       return std::max(a, b);
     }

@@ -42,8 +42,9 @@ struct VerifyPlan {
   bool wide;            // more segments per unit than one staged merge round holds
 };
 bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan);
-// What a workspace for blocks of up to n_q queries holds beside its header: a block small enough
-// for verify_kernel may need more partials than a longer one on verify_tc_kernel.
+// What a workspace for blocks of up to n_q queries holds beside its header.  A shorter block may need more
+// partials than a longer one: on either side of 24 query rows the kernels differ, past 256 and 512 rows
+// there are more, smaller units with fewer segments each, and at a tile's end the ranges are cut anew.
 size_t verify_region_bytes(const bd_shape& s, int n_q);
 size_t verify_partials_bytes(const bd_shape& s, const VerifyPlan& plan);
 // q/o/lse as in bd_verify_attn; ws_region points at the op region, counters/status into ws.
@@ -84,6 +85,14 @@ struct LsePlan {
   size_t smem_bytes, part_bytes;
 };
 bool lse_plan(const bd_shape& s, int window, LsePlan* plan);
+// The context whose last n_q positions are the block's rows.
+inline bd_shape block_context(const bd_shape& s, int n_q) {
+  bd_shape ls = s;
+  ls.t_ctx = s.t_ctx + n_q;
+  return ls;
+}
+// The same for a block without an output of up to n_q queries behind a context of s.t_ctx.
+size_t lse_region_bytes(const bd_shape& s, int n_q);
 // len_offset is added to every sequence's length (seq_lens); part: plan.part_bytes of scratch.
 cudaError_t launch_lse(const bd_shape& s, const LsePlan& plan, const void* k_cache, const void* q, int window,
                        int len_offset, bool window_ready, float* lse_out, void* part, int* counters, int* status,

@@ -1515,6 +1515,15 @@ bool lse_plan(const bd_shape& s, int window, LsePlan* plan) {
   return plan->smem_bytes <= 227 * 1024;
 }
 
+size_t lse_region_bytes(const bd_shape& s, int n_q) {
+  size_t bytes = 0;
+  for (int n = 1; n <= n_q; ++n) {
+    LsePlan lp;
+    if (lse_plan(block_context(s, n), n, &lp)) bytes = std::max(bytes, lp.part_bytes);
+  }
+  return bytes;
+}
+
 cudaError_t launch_lse(const bd_shape& s, const LsePlan& plan, const void* k_cache, const void* q, int window,
                        int len_offset, bool window_ready, float* lse_out, void* part, int* counters, int* status,
                        cudaStream_t stream) {

@@ -468,10 +468,9 @@ size_t verify_partials_bytes(const bd_shape& s, const VerifyPlan& plan) {
 
 size_t verify_region_bytes(const bd_shape& s, int n_q) {
   size_t bytes = 0;
-  for (const int rows : {INT_MAX, kVMaxRows, kVTcRows}) {
-    const int n = std::min(n_q, rows / (s.h_q / s.h_kv));
+  for (int n = 1; n <= n_q; ++n) {
     VerifyPlan vp;
-    if (n >= 1 && verify_plan(s, n, &vp)) bytes = std::max(bytes, verify_partials_bytes(s, vp));
+    if (verify_plan(s, n, &vp)) bytes = std::max(bytes, verify_partials_bytes(s, vp));
   }
   return bytes;
 }
