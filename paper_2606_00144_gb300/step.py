@@ -78,21 +78,22 @@ class SpecStep:
         The window rows form a verify block that starts W positions before the context's
         end.  With per-sequence lengths, sequence b's rows sit at seq_lens[b] - W ..
         seq_lens[b] - 1, so every length must exceed the window W."""
-        lens = None
-        if self.seq_lens is not None:
-            ts = torch.cuda.ExternalStream(stream) if isinstance(stream, int) else \
-                (stream or torch.cuda.current_stream())
-            with torch.cuda.stream(ts):
-                lens = torch.sub(self.seq_lens, self.window)          # where each window block starts
-            lens.record_stream(ts)
-        sh = B.make_shape(self.shape.batch, self.shape.h_q, self.shape.h_kv, self.shape.head_dim,
-                          self.shape.t_ctx - self.window, self.shape.t_cap, lens)
-        if out is None:
-            out = torch.empty(self.shape.batch, self.shape.h_q, self.window, dtype=torch.float32,
-                              device=k_cache.device)
-        # (a workspace of this call's own; its size covers a block with an output too, 17 MB for 64
-        # units of 16K, so only the words that have to be zero are filled)
-        ws = B.Workspace(B.bd_workspace_size(sh, B.BD_OP_VERIFY, 1, self.window), k_cache.device,
-                         units=sh.batch * sh.h_kv)
+        # what the call allocates belongs to the stream it runs on: filled, used and given back in its order
+        ts = torch.cuda.ExternalStream(stream) if isinstance(stream, int) else stream
+        caller = torch.cuda.current_stream() if ts is not None and out is None else None
+        with torch.cuda.stream(ts):
+            # with per-sequence lengths: where each window block starts
+            lens = None if self.seq_lens is None else torch.sub(self.seq_lens, self.window)
+            sh = B.make_shape(self.shape.batch, self.shape.h_q, self.shape.h_kv, self.shape.head_dim,
+                              self.shape.t_ctx - self.window, self.shape.t_cap, lens)
+            if out is None:
+                out = torch.empty(self.shape.batch, self.shape.h_q, self.window, dtype=torch.float32,
+                                  device=k_cache.device)
+            # (a workspace of this call's own; its size covers a block with an output too, 17 MB for 64
+            # units of 16K, so only the words that have to be zero are filled)
+            ws = B.Workspace(B.bd_workspace_size(sh, B.BD_OP_VERIFY, 1, self.window), k_cache.device,
+                             units=sh.batch * sh.h_kv)
+        if caller is not None:
+            out.record_stream(caller)
         B.bd_verify_attn(sh, q_win, self.window, k_cache, None, None, out, ws, stream)
         return out
