@@ -78,22 +78,30 @@ class SpecStep:
         The window rows form a verify block that starts W positions before the context's
         end.  With per-sequence lengths, sequence b's rows sit at seq_lens[b] - W ..
         seq_lens[b] - 1, so every length must exceed the window W."""
+        if stream is None:
+            return self._window_lse(k_cache, q_win, out, None)
         # what the call allocates belongs to the stream it runs on: filled, used and given back in its order
         ts = torch.cuda.ExternalStream(stream) if isinstance(stream, int) else stream
-        caller = torch.cuda.current_stream() if ts is not None and out is None else None
+        caller = torch.cuda.current_stream()
         with torch.cuda.stream(ts):
-            # with per-sequence lengths: where each window block starts
-            lens = None if self.seq_lens is None else torch.sub(self.seq_lens, self.window)
-            sh = B.make_shape(self.shape.batch, self.shape.h_q, self.shape.h_kv, self.shape.head_dim,
-                              self.shape.t_ctx - self.window, self.shape.t_cap, lens)
-            if out is None:
-                out = torch.empty(self.shape.batch, self.shape.h_q, self.window, dtype=torch.float32,
-                                  device=k_cache.device)
-            # (a workspace of this call's own; its size covers a block with an output too, 17 MB for 64
-            # units of 16K, so only the words that have to be zero are filled)
-            ws = B.Workspace(B.bd_workspace_size(sh, B.BD_OP_VERIFY, 1, self.window), k_cache.device,
-                             units=sh.batch * sh.h_kv)
-        if caller is not None:
-            out.record_stream(caller)
+            result = self._window_lse(k_cache, q_win, out, stream)
+        if out is None:
+            result.record_stream(caller)
+        return result
+
+    def _window_lse(self, k_cache, q_win, out, stream):
+        s = self.shape
+        # with per-sequence lengths: where each window block starts
+        lens = None if self.seq_lens is None else torch.sub(self.seq_lens, self.window)
+        sh = B.make_shape(s.batch, s.h_q, s.h_kv, s.head_dim, s.t_ctx - self.window, s.t_cap, lens)
+        if out is None:
+            out = torch.empty(s.batch, s.h_q, self.window, dtype=torch.float32, device=k_cache.device)
+        # A workspace of this call's own.  A selection of the whole context ranks nothing and needs room for
+        # these same normalisers, some hundred KB; sized for a verify block it would be planned for with an
+        # output too (17 MB for 64 units of 16K), which for a small context takes longer than the kernel.
+        # A small one is filled as a whole (one call), of a large one only the words that have to be zero.
+        size = B.bd_workspace_size(s, B.BD_OP_SELECT, s.t_ctx, self.window) or \
+            B.bd_workspace_size(sh, B.BD_OP_VERIFY, 1, self.window)
+        ws = B.Workspace(size, k_cache.device, units=s.batch * s.h_kv if size > 1 << 20 else None)
         B.bd_verify_attn(sh, q_win, self.window, k_cache, None, None, out, ws, stream)
         return out
