@@ -406,14 +406,17 @@ struct LseParams {
   int len_offset;            // added to every length (a verify block ends n_q past its context)
   int h_kv, units;
 };
-constexpr int kLMaxSeg = 8;      // segments of one unit with per-sequence lengths (bounds the partials)
+// Segments of one unit with per-sequence lengths (bounds the partials): 33 while the units are not many
+// times the SMs, since all but a few sequences may be short.  (One sequence of 64K, 8 units of 24 or 32 rows:
+// 53.5 us with 8 segments.)
+constexpr int kLMinSeg = 8, kLMaxSeg = 33;
 constexpr int kLThreads = 320;   // producer, MMA, eight epilogue warps (two per TMEM lane quarter)
 constexpr int kLAcc = 4;         // TMEM accumulators of 128 columns
 constexpr int kLStages = 4;
 
 // RAGGED: per-sequence lengths; every CTA lays out the units' tiles itself (a prefix table in
 // shared memory, as score_kernel's ragged instance does) and the range per CTA is at least
-// tiles_per_cta, which keeps a unit within kLMaxSeg segments.
+// tiles_per_cta, which keeps a unit within max_seg segments.
 template <int D, bool RAGGED>
 __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParams p,
                                                                   const __grid_constant__ CUtensorMap kmap,
@@ -1494,10 +1497,10 @@ bool lse_plan(const bd_shape& s, int window, LsePlan* plan) {
   int max_seg = 1;
   if (s.seq_lens) {
     // the lengths are read on the device: every SM gets a CTA, and the range per CTA is
-    // bounded below so that a unit of tpu tiles spans at most kLMaxSeg ranges
+    // bounded below so that a unit of tpu tiles spans at most max_seg ranges
     grid = current_sm_count();
-    tpc = (tpu + kLMaxSeg - 2) / (kLMaxSeg - 1);
-    max_seg = kLMaxSeg;
+    max_seg = (int)std::min<long>(kLMaxSeg, std::max<long>(kLMinSeg, (long)kLMaxSeg * grid / units));
+    tpc = (tpu + max_seg - 2) / (max_seg - 1);
   } else {
     grid = (int)((total + tpc - 1) / tpc);
     for (long u = 0; u < std::min<long>(units, tpc); ++u)   // (the offsets repeat after tpc units)
