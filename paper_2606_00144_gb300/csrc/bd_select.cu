@@ -389,9 +389,10 @@ __global__ void __launch_bounds__(kSThreads, 1) score_kernel(const ScoreParams p
 // 4-stage ring) and the unit's rows (two buffers), warp 1 issues the MMAs into four TMEM
 // accumulators, warps 2-9 reduce (two warps per TMEM lane quarter).  A unit split over
 // several CTAs merges the segments' (max, sum) pairs in the CTA that finishes it last.
-// HBM-bound: 268 MB of K (64 units of 16K, 128 rows each) in about 50.8 us, 5.3 TB/s; the same rows as
-// an mma.sync verify block without V took 126.9 us, bound by the tensor pipe.  (Skipping the TMEM
-// quarters past nq_rows made the full 128-row case 1 us slower and is left out.)
+// HBM-bound: 268 MB of K (64 units of 16K, 128 rows each) in 46.5 us, 5.8 TB/s; the same rows as
+// an mma.sync verify block without V took 124 us, bound by the tensor pipe.  With up to 64 rows the
+// operand holds them two or four times (COPIES): 128 units of 16K, 32 rows, d 64 68.3 us with one copy
+// (one lane quarter computes all the exponentials that count), 48.6 with four; d 128 82.1 / 78.9.
 struct LseParams {
   const __nv_bfloat16* q_win;   // [units * nq_rows][D] (read by TMA; prefetched through this pointer)
   float* lse;          // [units * nq_rows] natural log
@@ -417,7 +418,20 @@ constexpr int kLStages = 4;
 // RAGGED: per-sequence lengths; every CTA lays out the units' tiles itself (a prefix table in
 // shared memory, as score_kernel's ragged instance does) and the range per CTA is at least
 // tiles_per_cta, which keeps a unit within max_seg segments.
-template <int D, bool RAGGED>
+constexpr float kLn2Rest = -1.9046542e-9f;   // ln 2 less kLn2
+// log(2^m l) for a whole number m: the logarithm of l's fraction alone is rounded before the last sum (that
+// of l itself, 5 or so, by half as much as the result).
+__device__ __forceinline__ float row_lse(float m, float l) {
+  if (!(l > 0.f)) return -INFINITY;
+  int e;
+  const float f = frexpf(l, &e);
+  const float x = m + (float)e;
+  return fmaf(x, kLn2, fmaf(x, kLn2Rest, logf(f)));
+}
+
+// COPIES: how often the unit's rows (at most 128 / COPIES) lie in the A operand, each copy taking its share
+// of a tile's columns: a quarter of the lanes holding all the rows would have all the exponentials.
+template <int D, bool RAGGED, int COPIES>
 __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParams p,
                                                                   const __grid_constant__ CUtensorMap kmap,
                                                                   const __grid_constant__ CUtensorMap qmap) {
@@ -426,6 +440,8 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
   constexpr uint32_t KTILE = kSKeys * D * 2;
   constexpr uint32_t QHALF = 128 * 128;      // one 64-column half of the 128 window rows
   constexpr uint32_t QTILE = 128 * D * 2;
+  constexpr int ROWS = 128 / COPIES;         // rows of a copy
+  constexpr int COLS = 64 / COPIES;          // columns of a tile per epilogue thread
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem);
@@ -570,14 +586,17 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
         const int qs = qcount & 1;
         bool ok = true;
         if (lane == 0) {
-          // rows unit*nq_rows .. +127 (past nq_rows: the next unit's rows or zero fill, whose
+          // rows unit*nq_rows .. + ROWS - 1 (past nq_rows: the next unit's rows or zero fill, whose
           // results are discarded)
           if (qcount >= 2) ok = mbar_wait(&qempty_bar[qs], ((qcount >> 1) - 1) & 1, p.status, abort_flag);
           if (ok) {
             uint8_t* qb = qbuf + qs * QTILE;
             mbar_arrive_expect_tx(&qfull_bar[qs], QTILE);
 #pragma unroll
-            for (int h = 0; h < D / 64; ++h) tma_load_2d(qb + h * QHALF, &qmap, &qfull_bar[qs], 64 * h, unit * p.nq_rows);
+            for (int h = 0; h < D / 64; ++h)
+#pragma unroll
+              for (int c = 0; c < COPIES; ++c)
+                tma_load_2d(qb + h * QHALF + c * ROWS * 128, &qmap, &qfull_bar[qs], 64 * h, unit * p.nq_rows);
           }
         }
         if (!__shfl_sync(0xffffffffu, ok, 0)) break;
@@ -626,12 +645,13 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
     tc_commit(lead, drain_bar);
     mbar_wait(drain_bar, 0, p.status, nullptr);
   } else {
-    // ---------------------------------------------------------------- epilogue: a row's half per thread
+    // ---------------------------------------------------------------- epilogue: COLS columns of a row per thread
     grid_dependency_wait();
     allow_dependent_launch();
     const int quad = warp & 3;                  // TMEM lanes quad*32 .. quad*32+31
     const int half = (warp - 2) >> 2;           // warps 2-5: columns 0-63, warps 6-9: 64-127
-    const int row = quad * 32 + lane;
+    const int copy = quad * 32 / ROWS, row = quad * 32 + lane - copy * ROWS;
+    const bool first_copy = half == 0 && copy == 0;       // merges and writes its row
     int pw = p.t_ctx - p.window + row % p.window;         // last key the row sees
     int first_masked = p.t_ctx - p.window;                // keys past it are hidden from some row
     int cur_unit = -1, unit = unit_first;
@@ -659,31 +679,38 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
         const bool masked = key0 + kSKeys - 1 > first_masked;
         const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 128);
         {
-          const int c0 = 64 * half;
-          float v[64];
-          tc_ld_32cols(taddr + c0, *reinterpret_cast<float(*)[32]>(&v[0]));
-          tc_ld_32cols(taddr + c0 + 32, *reinterpret_cast<float(*)[32]>(&v[32]));
+          const int c0 = 64 * half + COLS * copy;
+          float v[COLS];
+          if constexpr (COLS == 16) {
+            tc_ld_16cols(taddr + c0, v);
+          } else {
+#pragma unroll
+            for (int j = 0; j < COLS; j += 32) tc_ld_32cols(taddr + c0 + j, *reinterpret_cast<float(*)[32]>(&v[j]));
+          }
           tc_wait_ld();
           if (masked) {
 #pragma unroll
-            for (int j = 0; j < 64; ++j) v[j] = key0 + c0 + j <= pw ? v[j] : -INFINITY;
+            for (int j = 0; j < COLS; ++j) v[j] = key0 + c0 + j <= pw ? v[j] : -INFINITY;
           }
           float mx0 = fmaxf(v[0], v[1]), mx1 = fmaxf(v[2], v[3]);
 #pragma unroll
-          for (int j = 4; j < 64; j += 4) {
+          for (int j = 4; j < COLS; j += 4) {
             mx0 = fmaxf(mx0, fmaxf(v[j], v[j + 1]));
             mx1 = fmaxf(mx1, fmaxf(v[j + 2], v[j + 3]));
           }
           const float mxs = fmaxf(mx0, mx1) * p.scale_log2;
           if (mxs > m) {
-            l *= fast_exp2(m - mxs);                 // m = -inf: l is still 0
-            m = mxs;
+            // rounded up to a whole number, so that sums under different maxima meet by exact powers of two
+            // (by additions: ceilf shares a unit with the exponentials, 39.4 us for 64 units of 16K, d 64, against 38.9)
+            const float up = __fadd_ru(mxs, 12582912.f) - 12582912.f;
+            l *= fast_exp2(m - up);                  // m = -inf: l is still 0
+            m = up;
           }
           const float2 cc = make_float2(p.scale_log2, p.scale_log2);
           const float2 nm = make_float2(m == -INFINITY ? 0.f : -m, m == -INFINITY ? 0.f : -m);
           float2 a0 = make_float2(0.f, 0.f), a1 = a0;
 #pragma unroll
-          for (int j = 0; j < 64; j += 4) {
+          for (int j = 0; j < COLS; j += 4) {
             const float2 x0 = ffma2(make_float2(v[j], v[j + 1]), cc, nm);
             const float2 x1 = ffma2(make_float2(v[j + 2], v[j + 3]), cc, nm);
             a0 = fadd2(a0, make_float2(fast_exp2(x0.x), fast_exp2(x0.y)));
@@ -697,20 +724,23 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
       }
       if (i != n - 1 && g + 1 != unit_end(unit)) continue;
       // ------------------------------------------------------------ end of this CTA's part of the unit
-      // the two column halves of each row meet first
-      ml_s[half * 128 + row] = alive ? make_float2(m, l) : make_float2(-INFINITY, 0.f);
+      // a row's column shares meet first
+      ml_s[(half * COPIES + copy) * ROWS + row] = alive ? make_float2(m, l) : make_float2(-INFINITY, 0.f);
       named_bar(1, 256);
       const int c_first = unit_begin(unit) / tpc, c_last = (unit_end(unit) - 1) / tpc;
       const int n_seg = c_last - c_first + 1;
       const size_t row0 = (size_t)unit * p.nq_rows;
       float2* seg = p.part + (size_t)unit * p.max_seg * 128;
-      if (half == 0) {
-        const float2 o = ml_s[128 + row];
-        const float M2 = fmaxf(m, o.x);
-        l = (m == -INFINITY ? 0.f : l * fast_exp2(m - M2)) + (o.x == -INFINITY ? 0.f : o.y * fast_exp2(o.x - M2));
-        m = M2;
+      if (first_copy) {
+#pragma unroll
+        for (int h = 1; h < 2 * COPIES; ++h) {
+          const float2 o = ml_s[h * ROWS + row];
+          const float M2 = fmaxf(m, o.x);
+          l = (m == -INFINITY ? 0.f : l * fast_exp2(m - M2)) + (o.x == -INFINITY ? 0.f : o.y * fast_exp2(o.x - M2));
+          m = M2;
+        }
         if (n_seg == 1) {
-          if (alive && row < p.nq_rows) p.lse[row0 + row] = l > 0.f ? fmaf(m, kLn2, logf(l)) : -INFINITY;
+          if (alive && row < p.nq_rows) p.lse[row0 + row] = row_lse(m, l);
         } else if (alive) {
           seg[(size_t)((int)blockIdx.x - c_first) * 128 + row] = make_float2(m, l);
         }
@@ -718,9 +748,9 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
       if (n_seg > 1) {
         __threadfence();
         named_bar(1, 256);
-        if (half == 0 && row == 0) *last_flag = alive && atomicAdd(&p.counters[unit], 1) == n_seg - 1;
+        if (first_copy && row == 0) *last_flag = alive && atomicAdd(&p.counters[unit], 1) == n_seg - 1;
         named_bar(1, 256);
-        if (half == 0 && *last_flag) {
+        if (first_copy && *last_flag) {
           __threadfence();
           float M = -INFINITY;
           for (int k = 0; k < n_seg; ++k) M = fmaxf(M, __ldcg(&seg[(size_t)k * 128 + row].x));
@@ -729,7 +759,7 @@ __global__ void __launch_bounds__(kLThreads, 1) window_lse_kernel(const LseParam
             const float2 ml = __ldcg(&seg[(size_t)k * 128 + row]);
             L += ml.x == -INFINITY ? 0.f : ml.y * fast_exp2(ml.x - M);
           }
-          if (row < p.nq_rows) p.lse[row0 + row] = L > 0.f ? fmaf(M, kLn2, logf(L)) : -INFINITY;
+          if (row < p.nq_rows) p.lse[row0 + row] = row_lse(M, L);
           if (row == 0) p.counters[unit] = 0;
         }
       }
@@ -1527,6 +1557,9 @@ size_t lse_region_bytes(const bd_shape& s, int n_q) {
   return bytes;
 }
 
+// As many copies of a unit's rows as the 128-row operand holds, of 1, 2 and 4 (see window_lse_kernel).
+static int lse_copies(int nq_rows) { return nq_rows <= 32 ? 4 : nq_rows <= 64 ? 2 : 1; }
+
 cudaError_t launch_lse(const bd_shape& s, const LsePlan& plan, const void* k_cache, const void* q, int window,
                        int len_offset, bool window_ready, float* lse_out, void* part, int* counters, int* status,
                        cudaStream_t stream) {
@@ -1534,7 +1567,8 @@ cudaError_t launch_lse(const bd_shape& s, const LsePlan& plan, const void* k_cac
   CUtensorMap kmap, qmap;
   cudaError_t err = make_cache_map(&kmap, k_cache, units, s.t_cap, s.t_ctx, s.head_dim, kSKeys);
   if (err != cudaSuccess) return err;
-  err = make_rows_map(&qmap, q, (long long)units * plan.nq_rows, s.head_dim, 128);
+  const int copies = lse_copies(plan.nq_rows);
+  err = make_rows_map(&qmap, q, (long long)units * plan.nq_rows, s.head_dim, 128 / copies);
   if (err != cudaSuccess) return err;
   LseParams p;
   p.q_win = static_cast<const __nv_bfloat16*>(q);
@@ -1556,10 +1590,13 @@ cudaError_t launch_lse(const bd_shape& s, const LsePlan& plan, const void* k_cac
   p.h_kv = s.h_kv;
   p.units = units;
   p.scale_log2 = kLog2e / sqrtf((float)s.head_dim);
-  void* fn = s.seq_lens ? (s.head_dim == 64 ? reinterpret_cast<void*>(&window_lse_kernel<64, true>)
-                                            : reinterpret_cast<void*>(&window_lse_kernel<128, true>))
-                        : (s.head_dim == 64 ? reinterpret_cast<void*>(&window_lse_kernel<64, false>)
-                                            : reinterpret_cast<void*>(&window_lse_kernel<128, false>));
+  void* fn = nullptr;
+#define BD_LSE(DD, R, C) \
+  if (s.head_dim == DD && (s.seq_lens != nullptr) == R && copies == C) fn = reinterpret_cast<void*>(&window_lse_kernel<DD, R, C>);
+  BD_LSE(64, false, 1) BD_LSE(64, false, 2) BD_LSE(64, false, 4) BD_LSE(64, true, 1) BD_LSE(64, true, 2) BD_LSE(64, true, 4)
+  BD_LSE(128, false, 1) BD_LSE(128, false, 2) BD_LSE(128, false, 4) BD_LSE(128, true, 1) BD_LSE(128, true, 2)
+  BD_LSE(128, true, 4)
+#undef BD_LSE
   err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
   if (err != cudaSuccess) return err;
   void* args[] = {&p, &kmap, &qmap};
