@@ -1542,8 +1542,12 @@ bool lse_plan(const bd_shape& s, int window, LsePlan* plan) {
   plan->tiles_per_cta = tpc;
   plan->grid = grid;
   plan->max_seg = max_seg;
-  plan->smem_bytes = 2048 + (size_t)2 * 128 * s.head_dim * 2 + (size_t)kLStages * kSKeys * s.head_dim * 2 +
-                     2 * 128 * sizeof(float2) + (s.seq_lens ? align_up((size_t)(units + 1) * 4, 16) : 0);
+  // (at least what keeps a second CTA off the SM: it would wait for the first one's tensor memory while, with
+  // the preceding kernel still on some SMs, others hold none.  A self-mode selection of 64 units of 16K, d 64:
+  // 110 us with two CTAs to an SM, 76 with one.)
+  const size_t smem = 2048 + (size_t)2 * 128 * s.head_dim * 2 + (size_t)kLStages * kSKeys * s.head_dim * 2 +
+                      2 * 128 * sizeof(float2) + (s.seq_lens ? align_up((size_t)(units + 1) * 4, 16) : 0);
+  plan->smem_bytes = std::max<size_t>(smem, 114 * 1024);
   plan->part_bytes = max_seg > 1 ? align_up((size_t)units * max_seg * 128 * sizeof(float2), 256) : 0;
   return plan->smem_bytes <= 227 * 1024;
 }
