@@ -387,7 +387,7 @@ cudaError_t launch_advance(const bd_shape& s, int window, int n_q, const int32_t
   p.capacity = capacity;
   const size_t smem = advance_smem(window, s.head_dim);
   void* fn = s.head_dim == 64 ? reinterpret_cast<void*>(&advance_kernel<64>) : reinterpret_cast<void*>(&advance_kernel<128>);
-  cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = allow_shared_memory(fn, sizeof(int) * kVThreads / 32);
   if (err != cudaSuccess) return err;
   void* args[] = {&p};
   return launch_kernel(fn, dim3(s.h_q, s.batch), dim3(kVThreads), smem, stream, args, 0);

@@ -38,6 +38,7 @@ constexpr int kDRows = 80;        // rows per shared-memory tile: sub-tiles of 1
 constexpr int kDLongRows = 160;   // the same for long slices (LONG instances)
 constexpr int kDMaxCluster = 8;   // CTAs of a cluster: the portable cluster size
 constexpr int kDMaxParts = 8;     // clusters per unit
+constexpr size_t kDLongStatic = 16;   // bytes of static shared memory of a LONG instance, rounded up
 
 struct DraftParams {
   const __nv_bfloat16* q;      // [units * g][D]
@@ -405,7 +406,7 @@ static long clusters_held(int d, int g_kernel, bool longs, int c) {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_shared_memory(fn, longs ? kDLongStatic : 0) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
       n = per_sm * current_sm_count() / c;
@@ -472,14 +473,14 @@ bool draft_plan(const bd_shape& s, int budget, int n_steps, size_t room, DraftPl
       lp.rows_per_split = (int)rps;
       lp.longs = true;
       if (draft_partials_bytes(s, lp) > room ||
-          smem_bytes(s.head_dim, g_kernel, true, 2, c, draft_pos_slots(lp)) > 227 * 1024)
+          smem_bytes(s.head_dim, g_kernel, true, 2, c, draft_pos_slots(lp)) > kMaxSmem - kDLongStatic)
         continue;
       *plan = lp;
       best_us = us;
     }
   }
-  return smem_bytes(s.head_dim, g_kernel, plan->longs, draft_stages(*plan, units), plan->n_split, draft_pos_slots(*plan)) <=
-         227 * 1024;
+  return plan->longs || smem_bytes(s.head_dim, g_kernel, false, draft_stages(*plan, units), plan->n_split,
+                                   draft_pos_slots(*plan)) <= kMaxSmem;
 }
 
 cudaError_t launch_draft(const bd_shape& s, const DraftPlan& plan, const void* q, const void* k_cache,
@@ -516,8 +517,7 @@ cudaError_t launch_draft(const bd_shape& s, const DraftPlan& plan, const void* q
   p.g = g;
   void* fn = pick(s.head_dim, g_kernel, plan.longs);
   const size_t smem = smem_bytes(s.head_dim, g_kernel, plan.longs, p.n_stage, plan.n_split, p.pos_slots);
-  if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = allow_shared_memory(fn, plan.longs ? kDLongStatic : 0);
   if (err != cudaSuccess) return err;
 
   void* args[] = {&p};

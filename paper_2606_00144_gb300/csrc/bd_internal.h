@@ -20,6 +20,14 @@ int current_sm_count();   // SMs of the current device (cached per device)
 cudaError_t launch_kernel(const void* fn, dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                           void** args, int cluster_x);
 
+// Shared memory a CTA may have, and permission for `fn` to ask for all of it beside static_bytes of its
+// own.  The permission belongs to the function, not to a launch: set to each launch's own size, a thread
+// could lower it between another one's setting and launching.
+constexpr size_t kMaxSmem = 227 * 1024;
+inline cudaError_t allow_shared_memory(const void* fn, size_t static_bytes = 0) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem - static_bytes));
+}
+
 // ---------------------------------------------------------------------------- workspace
 // [0, 256): status word; [256, 256 + units*4 rounded to 256): per-unit arrival counters;
 // then the op-specific region.

@@ -1601,7 +1601,7 @@ cudaError_t launch_lse(const bd_shape& s, const LsePlan& plan, const void* k_cac
   BD_LSE(128, false, 1) BD_LSE(128, false, 2) BD_LSE(128, false, 4) BD_LSE(128, true, 1) BD_LSE(128, true, 2)
   BD_LSE(128, true, 4)
 #undef BD_LSE
-  err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
+  err = allow_shared_memory(fn);
   if (err != cudaSuccess) return err;
   void* args[] = {&p, &kmap, &qmap};
   return launch_kernel(fn, dim3(plan.grid), dim3(kLThreads), plan.smem_bytes, stream, args, 0);
@@ -1693,7 +1693,7 @@ cudaError_t launch_select(const bd_shape& s, const SelectPlan& plan, const void*
     p.h_kv = s.h_kv;
     p.window_ready = (flags & BD_SELECT_WINDOW_READY) ? 1 : 0;
     void* fn = score_fn(s.head_dim, plan.nq_pad, s.seq_lens != nullptr).fn;
-    err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
+    err = allow_shared_memory(fn);
     if (err != cudaSuccess) return err;
     void* args[] = {&p, &kmap, &qmap};
     err = launch_kernel(fn, dim3(plan.grid), dim3(kSThreads), plan.smem_bytes, stream, args, 0);
@@ -1735,7 +1735,7 @@ cudaError_t launch_select(const bd_shape& s, const SelectPlan& plan, const void*
   if (!plan.keep_all && plan.need_scores && chunk == 1 && plan.n_mid <= kLeanMaxItems && 4L * units > sms) {
     const size_t smem = (size_t)align_up(plan.n_mid, 4) * 4;
     void* fn = reinterpret_cast<void*>(&topk_token_kernel);
-    err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    err = allow_shared_memory(fn, 64 * 1024);   // (its own arrays: 34 KB)
     if (err != cudaSuccess) return err;
     return launch_kernel(fn, dim3(units), dim3(kTopkThreads), smem, stream, targs, 0);
   }

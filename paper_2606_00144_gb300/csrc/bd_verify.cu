@@ -371,8 +371,9 @@ int occupancy(const KernelInfo& k) {
   cudaGetDevice(&dev);
   if (k.fn == last_fn && dev == last_dev) return last_occ;
   int occ = 1;
-  cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, kVThreads, k.smem) != cudaSuccess || occ < 1) occ = 1;
+  if (allow_shared_memory(k.fn) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, kVThreads, k.smem) != cudaSuccess || occ < 1)
+    occ = 1;
   (void)cudaGetLastError();
   last_fn = k.fn;
   last_dev = dev;
@@ -511,7 +512,7 @@ cudaError_t launch_verify(const bd_shape& s, const VerifyPlan& plan, int n_q, co
   p.tile_rows = plan.q_tiles == 2 ? (plan.nq_rows + 1) / 2 : plan.nq_rows;
   const void* fn = plan.q_tiles ? verify_tc_fn(s.head_dim, plan.q_tiles, s.seq_lens != nullptr)
                                 : select_kernel(s.head_dim, plan.nt, s.seq_lens == nullptr, plan.wide).fn;
-  err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
+  err = allow_shared_memory(fn);
   if (err != cudaSuccess) return err;
   CUtensorMap qmap;
   if (plan.q_tiles) {
