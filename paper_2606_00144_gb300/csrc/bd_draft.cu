@@ -374,27 +374,28 @@ static int draft_pos_slots(const DraftPlan& plan) {
 // tile up to 8, two beyond).
 int draft_group_instance(int g) { return g <= 1 ? 1 : g <= 2 ? 2 : g <= 4 ? 4 : g <= 8 ? 8 : 16; }
 
-// Clusters of c CTAs that the device holds at once: LONG instances at one CTA per SM, short ones
-// with two tile buffers at two.  (A GPC's SMs are shared out by whole clusters, so it is fewer than the SMs' CTAs
-// divided by c.)
-static long clusters_held(int d, int g_kernel, bool longs, int c) {
+// CTAs of smem bytes that an SM's shared memory holds (228 KB, a CTA taking 1 KB more than it asks for).
+static int ctas_per_sm(size_t smem) { return (int)std::min<size_t>(4, 228 * 1024 / (smem + 1024)); }
+
+// Clusters of c CTAs of smem bytes that the device holds at once.  (A GPC's SMs are shared out by whole clusters,
+// so it is fewer than the SMs' CTAs divided by c.)  Kept per instance, c and CTAs an SM.
+static long clusters_held(int d, int g_kernel, bool longs, int c, size_t smem) {
   static thread_local int cache_dev = -1;
-  static thread_local int cache[2][kDMaxCluster + 1];
+  static thread_local int cache[2][2][17][kDMaxCluster + 1][5];
   int dev = 0;
-  const int per_sm = longs ? 1 : 2;
+  const int per_sm = ctas_per_sm(smem);
+  const long guess = (long)per_sm * current_sm_count() / c;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     (void)cudaGetLastError();
-    return per_sm * current_sm_count() / c;
+    return guess;
   }
   if (dev != cache_dev) {
-    for (auto& row : cache)
-      for (int& n : row) n = -1;
+    std::fill_n(&cache[0][0][0][0][0], sizeof(cache) / sizeof(int), -1);
     cache_dev = dev;
   }
-  int& held = cache[longs][c];
+  int& held = cache[longs][d == 128][g_kernel][c][per_sm];
   if (held < 0) {
     void* fn = pick(d, g_kernel, longs);
-    const size_t smem = (longs ? 200 : 100) * 1024;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c);
     cfg.blockDim = dim3(2 * (longs ? kDLongRows : kDRows));
@@ -409,7 +410,7 @@ static long clusters_held(int d, int g_kernel, bool longs, int c) {
     if (allow_shared_memory(fn, longs ? kDLongStatic : 0) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
-      n = per_sm * current_sm_count() / c;
+      n = (int)guess;
     }
     held = n;
   }
@@ -435,34 +436,51 @@ bool draft_plan(const bd_shape& s, int budget, int n_steps, size_t room, DraftPl
   const long entries = (long)budget + n_steps;
   const int g_kernel = draft_group_instance(g);
   // one tile per CTA up to a cluster of 8, but no more CTAs than one wave holds at the
-  // occupancy the slice's stage count gives (three single-stage or two double-buffered
-  // CTAs per SM, draft_stages): a second wave would repeat the pass's whole latency chain.  With
-  // two buffers counted in whole clusters: 48 units of 2K rows took 16.5 us a pass in clusters of six, some
-  // of which waited for a second wave, 11.4 in clusters of five; 40 units of 2K 14.5 / 9.9.
+  // occupancy the slice's stage count gives (up to three single-stage or two double-buffered
+  // CTAs per SM, draft_stages, fewer where rank 0's partials leave no room): a second wave would
+  // repeat the pass's whole latency chain.  With two buffers counted in whole clusters: 48 units of 2K rows
+  // took 16.5 us a pass in clusters of six, some of which waited for a second wave, 11.4 in clusters of five.
+  // With the launch's own shared memory: 32 units of 2K rows, groups of 8 21.4 us in clusters of eight (117 KB,
+  // one CTA to an SM), 9.4 in smaller ones; groups of 16 27.9 / 13.1, 48 units of 512 rows 14.3 / 10.3.
   const long units = (long)s.batch * s.h_kv;
   const long sms = current_sm_count();
-  int n_split = (int)std::min<long>((entries + kDRows - 1) / kDRows, kDMaxCluster);
+  const int most = (int)std::min<long>((entries + kDRows - 1) / kDRows, kDMaxCluster);
+  auto dbuf_of = [&](int n) {
+    const long rps = (entries + n - 1) / n;
+    return (rps > kDRows && units * n <= 2 * sms) || rps > 2 * kDRows;
+  };
+  auto smem_of = [&](int n) {   // the row table of a CTA's slice sits in shared memory beside its tiles
+    const long slots = ((entries + n - 1) / n + kDRows - 1) / kDRows * kDRows;
+    return smem_bytes(s.head_dim, g_kernel, false, dbuf_of(n) ? 2 : 1, n, (int)std::min<long>(slots, 1 << 24));
+  };
+  int n_split = most;
   for (; n_split > 1; --n_split) {
-    const long rps = (entries + n_split - 1) / n_split, ctas = units * n_split;
-    const bool dbuf = (rps > kDRows && ctas <= 2 * sms) || rps > 2 * kDRows;
-    if (ctas <= (dbuf ? 2 : 3) * sms && (!dbuf || units <= clusters_held(s.head_dim, g_kernel, false, n_split))) break;
+    const bool dbuf = dbuf_of(n_split);
+    const size_t smem = smem_of(n_split);
+    if (smem <= kMaxSmem && units * n_split <= std::min(dbuf ? 2 : 3, ctas_per_sm(smem)) * sms &&
+        (!dbuf || units <= clusters_held(s.head_dim, g_kernel, false, n_split, smem)))
+      break;
   }
   n_split = std::max(n_split, 1);
+  if (smem_of(n_split) > kMaxSmem) {   // a view whose table only wider clusters hold, in as many waves as it takes
+    for (n_split = most; n_split > 1 && smem_of(n_split) > kMaxSmem;) --n_split;
+  }
   const long rows_per_split = (entries + n_split - 1) / n_split;
   if (rows_per_split > (1L << 24)) return false;
   plan->rows_per_split = (int)rows_per_split;
   plan->n_split = n_split;
   plan->n_clusters = 1;
   plan->longs = false;
-  // the row table of a CTA's slice sits in shared memory beside its tiles
   // A LONG instance where its estimate is the shorter: a fixed cost, one per tile a CTA walks
-  // (both fitted to passes of 4 units of 1K to 8K rows), one where clusters meet in memory.  Per pass,
-  // d 128, short / LONG measured: 4 units of 1K rows 5.1 / 4.8 us, 2K 7.2 / 5.8, 8K 16.2 / 7.7; 8 units of
+  // (both fitted to passes of 4 units of 1K to 8K rows, d 128), one where clusters meet in memory.  Per pass,
+  // short / LONG measured: d 128, 4 units of 1K rows 5.1 / 4.8 us, 2K 7.2 / 5.8, 8K 16.2 / 7.7; 8 units of
   // 8K 16.4 / 10.6; 16 units of 1K 5.4 / 6.2 (stays short), 4K 11.9 / 10.6; 64 units of 2K 13.5 / 13.5 (the
-  // L2's rate; stays short).  Clusters of two CTAs gained nothing.
+  // L2's rate; stays short); groups of 16, 4 units of 2K 10.3 / 9.0, 8K 22.1 / 12.2, 16 units of 8K 43.2 / 22.0;
+  // d 64, 4 units of 2K 5.3 / 4.7, 8K 11.9 / 7.4, 16 units of 8K 13.5 / 11.9, groups of 16 18.5 / 13.9.  Clusters
+  // of two CTAs gained nothing.
   double best_us = 3.1 + 1.0 * ((rows_per_split + kDRows - 1) / kDRows);
   for (int c = kDMaxCluster; c >= 3; --c) {
-    const long cap = clusters_held(s.head_dim, g_kernel, true, c);
+    const long cap = clusters_held(s.head_dim, g_kernel, true, c, 200 * 1024);   // (one CTA an SM)
     for (int k = 1; k <= kDMaxParts && units * k <= cap; ++k) {
       const long rps = (entries + c * k - 1) / (c * k);
       const double us = 3.0 + 1.33 * ((rps + kDLongRows - 1) / kDLongRows) + (k > 1 ? 2.05 : 0.0);
