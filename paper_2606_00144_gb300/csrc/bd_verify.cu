@@ -386,12 +386,15 @@ int occupancy(const KernelInfo& k) {
 // Blocks that verify_kernel could take but verify_tc_kernel streams faster: a third n8 tile slows
 // every tile of keys in the one (8 rows 81.5 us, 24 rows 86.3 us for 64 units of 16K), while the other
 // costs the same up to 128 rows and wants a merge launch, which pays once the batch fills the SMs by itself.
-// verify_kernel / verify_tc_kernel, d 128, us: 64 units, 24 rows, of 1K 17.0 / 16.3, 4K 31.9 / 30.2, 16K 87.1 / 85.7;
-// 128 units, 21 rows, of 4K 51.4 / 49.0; 12 rows: 15.0 / 16.3, 29.8 / 29.9, 85.3 / 85.3; 32 units, 24 rows, of 16K 47.9 /
-// 49.4; d 64, 64 units of 16K 49.8 / 58.5; per-sequence lengths, 21 rows 48.2 / 48.4.
+// verify_kernel / verify_tc_kernel, d 128, us: 64 units, 24 rows, of 1K 17.1 / 15.9, 4K 31.2 / 29.3, 16K 86.5 / 85.2;
+// 128 units, 21 rows, of 4K 50.1 / 48.2, 16K 159.3 / 158.3; 12 rows: 15.0 / 16.3, 29.8 / 29.9, 85.3 / 85.3; 32 units, 24
+// rows, of 16K 47.9 / 49.4; d 64, 64 units of 16K 49.8 / 58.5; per-sequence lengths, 21 rows 48.2 / 48.4.  Three full
+// n8 tiles over more than a million keys in many units stay: 24 rows, 128 units of 16K 158.2 / 159.7, 160 of 8K 104.7 /
+// 105.3, 256 of 8K 159.5 / 161.4 (but 128 of 8K 86.5 / 85.8, 256 of 4K 88.1 / 87.6, 96 of 16K 122.2 / 121.9).
 static bool tc_streams_better(const bd_shape& s, int n_q) {
-  return s.head_dim == 128 && s.seq_lens == nullptr && 3L * s.batch * s.h_kv > current_sm_count() &&
-         (long)s.t_ctx + n_q >= 1024;
+  const long units = (long)s.batch * s.h_kv, keys = (long)s.t_ctx + n_q;
+  if (s.head_dim != 128 || s.seq_lens != nullptr || 3 * units <= current_sm_count() || keys < 1024) return false;
+  return s.h_q / s.h_kv * n_q <= 21 || units < 128 || units * keys < 5L << 18;
 }
 
 bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
