@@ -62,7 +62,7 @@ struct VerifySmem {
 // NT: n8 tiles of query rows; SUBS: 16-key sub-tiles of a tile per consumer warp.
 // UNIFORM: one shared context length; the other instances lay out per-sequence lengths.
 template <int D, int NT, int SUBS, bool UNIFORM, bool WIDE>
-__global__ void __launch_bounds__(kVThreads) verify_kernel(const VerifyParams p,
+__global__ void __launch_bounds__(kVThreads, D == 128 && NT == 1 ? 1 : 0) verify_kernel(const VerifyParams p,
                                                            const __grid_constant__ CUtensorMap kmap,
                                                            const __grid_constant__ CUtensorMap vmap) {
   using L = VerifySmem<D, NT>;
