@@ -394,7 +394,8 @@ cudaError_t launch_advance(const bd_shape& s, int window, int n_q, const int32_t
 }
 
 int argmax_cluster(int rows, int vocab) {
-  const int want = (4 * current_sm_count() + rows - 1) / std::max(1, rows);   // four CTAs an SM
+  // as many as one wave of four CTAs an SM holds
+  const int want = 4 * current_sm_count() / std::max(1, rows);
   const int by_size = (vocab + kAMinPerCta - 1) / kAMinPerCta;
   return std::max(1, std::min(kAMaxCluster, std::min(want, by_size)));
 }
