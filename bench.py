@@ -29,6 +29,7 @@ import ctypes
 import dataclasses
 import json
 import math
+import re
 import statistics
 import subprocess
 import time
@@ -45,6 +46,9 @@ from paper_2606_00144_gb300 import workload as W
 METRIC = "spec-step attention µs & HBM GB/s (% of ~8 TB/s) at 16K ctx, B=512, γ=5"
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6800.0
+# what the two verify kernels are built from (their profiles carry its hash)
+VERIFY_SOURCES = {"verify_tc_kernel": ("bd_verify_tc.cu", "bd_verify.cuh", "bd_common.cuh"),
+                  "verify_kernel": ("bd_verify.cu", "bd_verify.cuh", "bd_attn_warp.cuh", "bd_common.cuh")}
 
 
 # ----------------------------------------------------------------------------- bytes the method must read
@@ -206,14 +210,9 @@ class Step:
             self.lse.append(st.window_lse(inp.k_cache, inp.q_win) if sel_mode == "carry" else None)
         torch.cuda.synchronize()
 
-    def launches_per_step(self):
-        # selection: top-B only (B >= T), else score + top-B (+ the window-LSE pass in self mode)
-        if self.budget >= self.wl.t_ctx:
-            sel = 1
-        else:
-            sel = 2 + (1 if self.sel_mode == "self" else 0)
-        # the verify block: its kernel and the merge of its segments
-        return self.wl.layers * (sel + self.wl.gamma + 2)
+    def verify(self):
+        for st, inp in zip(self.steps, self.layers):
+            st.verify(inp.q_verify, inp.k_cache, inp.v_cache)
 
     def run(self, marks=None, select=True):
         """One step; marks = [select, draft, verify, end] timing events (or None).  With
@@ -238,9 +237,7 @@ class Step:
                 self.steps[l].draft(j, inp.q_draft[j], inp.k_cache, inp.v_cache, view_ready=ready)
         if marks:
             record(marks[2])
-        for l in L:
-            inp = self.layers[l]
-            self.steps[l].verify(inp.q_verify, inp.k_cache, inp.v_cache)
+        self.verify()
         if marks:
             record(marks[3])
 
@@ -255,6 +252,43 @@ def capture(fn, n):
                 fn(i)
     torch.cuda.current_stream().wait_stream(s)
     return g
+
+
+def captured_kernels(fn):
+    """Names of the library's kernels that fn() launches, in order, from the nodes of a capture of
+    it (which runs nothing): which ones a call takes is decided by its plan."""
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def check(call, *args):
+        code = getattr(cu, call)(*args)
+        if code != 0:
+            raise RuntimeError(f"{call} failed: {code}")
+
+    names = []
+    with torch.cuda.graph(torch.cuda.CUDAGraph()):
+        fn()
+        stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        status, ident, graph = ctypes.c_int(), ctypes.c_uint64(), ctypes.c_void_p()
+        deps, n_deps, n = ctypes.c_void_p(), ctypes.c_size_t(), ctypes.c_size_t()
+        check("cuStreamGetCaptureInfo_v2", stream, ctypes.byref(status), ctypes.byref(ident), ctypes.byref(graph),
+              ctypes.byref(deps), ctypes.byref(n_deps))
+        check("cuGraphGetNodes", graph, None, ctypes.byref(n))
+        nodes = (ctypes.c_void_p * n.value)()
+        check("cuGraphGetNodes", graph, nodes, ctypes.byref(n))
+        for node in nodes:
+            kind, name = ctypes.c_int(), ctypes.c_char_p()
+            check("cuGraphNodeGetType", ctypes.c_void_p(node), ctypes.byref(kind))
+            if kind.value != 0:                              # not a kernel
+                continue
+            # CUDA_KERNEL_NODE_PARAMS: the function first, or (word 7) the library's kernel
+            params = (ctypes.c_uint64 * 16)()
+            check("cuGraphKernelNodeGetParams_v2", ctypes.c_void_p(node), params)
+            call = "cuFuncGetName" if params[0] else "cuKernelGetName"
+            check(call, ctypes.byref(name), ctypes.c_void_p(params[0] or params[7]))
+            own = re.match(r"_ZN2bd(\d+)", name.value.decode())
+            if own:
+                names.append(name.value.decode()[own.end():own.end() + int(own.group(1))])
+    return names
 
 
 def timed_replays(graphs, world):
@@ -331,6 +365,8 @@ def gpu_arm(args):
     value = job_throughput(layer_bytes["total"], args.steps, world, ms)
     peak, peak_src = measured_hbm_peak()
     verify_launch_bytes = per["verify"]
+    verify_kernels = captured_kernels(step.verify)
+    verify_kernels = verify_kernels[:len(verify_kernels) // wl.layers]       # one layer's
     verify_us = phase_us["verify"] / wl.layers
     achieved = verify_launch_bytes / (verify_us * 1e-6) / 1e9
     line = {
@@ -362,7 +398,7 @@ def gpu_arm(args):
         "algorithmic_bytes_per_step": layer_bytes,
         "breakdown_us": {k: round(v, 2) for k, v in phase_us.items()},
         "roofline": {
-            "kernel": "verify_tc_kernel and its merge (bd_verify_attn)",
+            "kernel": "%s (bd_verify_attn)" % " and ".join(verify_kernels),
             "bound": "hbm",
             "achieved": round(achieved, 1),
             "peak": peak,
@@ -370,10 +406,11 @@ def gpu_arm(args):
             "unit": "GB/s",
             "frac": round(achieved / peak, 3),
             "bytes_per_launch": verify_launch_bytes,
-            "traffic": profiled_traffic("verify_tc_kernel", wl.name, ("bd_verify_tc.cu", "bd_verify.cuh", "bd_common.cuh")),
-            "traffic_source": "profiles/verify_tc_kernel_%s.md (ncu dram__bytes_read.sum + dram__bytes_write.sum)" % wl.name,
+            "traffic": profiled_traffic(verify_kernels[0], wl.name, VERIFY_SOURCES[verify_kernels[0]]),
+            "traffic_source": "profiles/%s_%s.md (ncu dram__bytes_read.sum + dram__bytes_write.sum)"
+                              % (verify_kernels[0], wl.name),
         },
-        "gpu_launches": step.launches_per_step() * args.steps,
+        "gpu_launches": len(captured_kernels(step.run)) * args.steps,
         "clocks": clocks,
     }
     # the oracle's processes start here (spawned: they import while the GPU lines below run)
@@ -436,7 +473,8 @@ def extras(step, args):
     us = time_per_step(lambda: step.run(select=False), n, gs)
     b = (per["draft"] + per["verify"]) * wl.layers
     out["amortized_step"] = {"us_per_step": round(us, 2), "GB/s": round(b / (us * 1e-6) / 1e9, 1),
-                             "bytes_per_step": b, "launches_per_step": wl.layers * (wl.gamma + 2)}
+                             "bytes_per_step": b,
+                             "launches_per_step": len(captured_kernels(lambda: step.run(select=False)))}
 
     # greedy acceptance (Eq. accept, Algorithm 2): arg max of every drafter pass and of the
     # verify block over a Llama-3 vocabulary, then the prefix test; synthetic bf16 logits
@@ -484,7 +522,7 @@ def extras(step, args):
         us = time_per_step(v.run, n, gs)
         pb = step_bytes(wl, step.budget, step.n_recent, "self")["total"] * wl.layers
         out["self_mode"] = {"us_per_step": round(us, 2), "GB/s": round(pb / (us * 1e-6) / 1e9, 1),
-                            "bytes_per_step": pb, "launches_per_step": v.launches_per_step()}
+                            "bytes_per_step": pb, "launches_per_step": len(captured_kernels(v.run))}
         del v
 
     # token-level budget sweep with a recent window of B/4 (B >= T keeps the whole context)
