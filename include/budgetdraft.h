@@ -44,8 +44,8 @@
  *     stream).  A call returns BD_OK or a negative bd_status after validating every
  *     argument on the host BEFORE any launch; a failed launch returns BD_ERR_CUDA.
  *   - Workspace: `ws` is a caller-owned device buffer of at least
- *     bd_workspace_size(...) bytes for that call.  It must be zero-filled once
- *     before its first use; calls that finish leave its counter words zero again,
+ *     bd_workspace_size(...) bytes for that call (bd_draft_attn also takes less).  It must be
+ *     zero-filled once before its first use; calls that finish leave its counter words zero again,
  *     so it can be reused without clearing.  Calls that share one workspace must
  *     be ordered (same stream, or synchronised).  Kernels record device-side
  *     errors (a bounded wait that ran out) in the workspace's status word, which
@@ -67,7 +67,7 @@ typedef enum bd_status {
   BD_ERR_INVALID_ARG = -1,  /* a null pointer, a size out of range, inconsistent shape  */
   BD_ERR_UNSUPPORTED = -2,  /* valid but not implemented (head_dim, too many queries)    */
   BD_ERR_MISALIGNED = -3,   /* a tensor pointer lacks the alignment its call requires    */
-  BD_ERR_WORKSPACE = -4,    /* ws is NULL or smaller than bd_workspace_size()            */
+  BD_ERR_WORKSPACE = -4,    /* ws is NULL or smaller than the call needs                  */
   BD_ERR_CUDA = -5,         /* a CUDA runtime call or a launch failed                    */
   BD_ERR_TIMEOUT = -6       /* device side: a bounded wait ran out (status word only)    */
 } bd_status;
@@ -175,10 +175,14 @@ enum {
  *   flags    0 or BD_DRAFT_VIEW_READY.
  *   o_out    bf16 [batch, h_q, d];  lse_out fp32 [batch, h_q] (may be NULL).
  * Constraints: step_j >= 0, t_ctx + step_j < t_cap, h_q / h_kv <= 16.  The budget + step_j + 1
- * entries are split over at most 8 CTAs, each holding the row table of its slice in shared
+ * entries of a (sequence, KV head) are split over a cluster of at most 8 CTAs, or, where few of
+ * them leave SMs free, over up to 8 clusters, each CTA holding the row table of its slice in shared
  * memory beside its tiles: at head_dim 128 views of up to about 165K (GQA group 16) to
- * 290K (group 1) entries, fewer when batch * h_kv fills the GPU; a larger view returns
- * BD_ERR_UNSUPPORTED.
+ * 290K (group 1) entries, at head_dim 64 310K to 375K, more with several clusters; a larger view
+ * returns BD_ERR_UNSUPPORTED.  Several clusters leave partials in ws and are used only where ws_bytes
+ * has room for them (bd_workspace_size(BD_OP_DRAFT) always has): a workspace of the header and the
+ * counters alone, 256 + 4 * batch * h_kv bytes rounded up to 256, is accepted and takes one
+ * cluster, which is slower for long views and sums in another order.
  */
 int bd_draft_attn(const bd_shape* shape, const void* q, const void* k_cache, const void* v_cache,
                   const int32_t* idx, const int32_t* count, int budget, int step_j, unsigned flags,
@@ -194,7 +198,7 @@ int bd_draft_attn(const bd_shape* shape, const void* q, const void* k_cache, con
  *
  * Arguments and results are those of bd_draft_attn with flags = 0, minus ws and ws_bytes.  The call
  * allocates nothing: its scratch (status word and per-(sequence, KV head) counters; the
- * drafter's split-K partials are merged inside each thread-block cluster) is a 4 MiB
+ * drafter's split-K partials are merged inside one thread-block cluster per view) is a 4 MiB
  * array inside the library's device image, which every GPU
  * that loads the library keeps until the process exits.  A shape whose scratch would not
  * fit returns BD_ERR_WORKSPACE before any launch.
@@ -228,8 +232,9 @@ int bd_draft_static_status(void* stream);
  *   o_out    bf16 [batch, h_q, n_q, d], or NULL to compute lse only (V not read);
  *   lse_out  fp32 [batch, h_q, n_q] (may be NULL when o_out is not).
  * Constraints: 1 <= n_q, t_ctx + n_q <= t_cap, (h_q/h_kv)*n_q <= 768 (<= 128 when
- * o_out is NULL).  A KV head's query rows beyond 96 are processed in up to eight chunks
- * of equal size that stream the same keys side by side.
+ * o_out is NULL).  A KV head's query rows beyond 256 are processed in up to three chunks
+ * of equal size that stream the same keys side by side.  Cache rows past a sequence's own
+ * block are never used: they may hold anything, NaN included.
  */
 int bd_verify_attn(const bd_shape* shape, const void* q, int n_q, const void* k_cache,
                    const void* v_cache, void* o_out, float* lse_out, void* ws, size_t ws_bytes,

@@ -15,8 +15,9 @@ namespace bd {
 int current_sm_count();   // SMs of the current device (cached per device)
 
 // Launch with programmatic dependent launch allowed (the kernel may be scheduled while
-// its predecessor finishes; every kernel of this library waits on the grid dependency
-// before touching its inputs) and, when cluster_x > 0, as clusters of cluster_x CTAs.
+// its predecessor finishes; every kernel of this library waits on the grid dependency before it
+// writes anything or reads what the predecessor may have written, and some read older rows of the
+// caches sooner) and, when cluster_x > 0, as clusters of cluster_x CTAs.
 cudaError_t launch_kernel(const void* fn, dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                           void** args, int cluster_x);
 

@@ -297,7 +297,6 @@ __global__ void __launch_bounds__(128) verify_merge_kernel(const float* o_part, 
     if (tid + 32 < n) w[tid + 32] = e1 * inv;
     if (tid == 0 && lse) lse[orow] = mx == -INFINITY ? -INFINITY : mx + logf(tot);
   }
-  if (o == nullptr) return;
   const int q = tid % Q, g = tid / Q;
   float4 v[PER];
 #pragma unroll

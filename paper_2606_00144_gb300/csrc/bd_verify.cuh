@@ -14,7 +14,8 @@ struct VerifyParams {
   const __nv_bfloat16* q;
   __nv_bfloat16* o;
   float* lse;
-  float* o_part;       // [units][max_seg][nq_rows][D]
+  float* o_part;       // [units][max_seg] partials of nq_rows x D floats: verify_kernel's [nq_rows][D],
+                       // verify_tc_kernel's [D/4][nq_rows] float4
   float* lse_part;     // [units][max_seg][nq_rows]
   int* counters;       // [units]
   int* nseg;           // [units] segments of each unit (wide plans: read by verify_merge_kernel)
