@@ -1555,6 +1555,7 @@ bool lse_plan(const bd_shape& s, int window, LsePlan* plan) {
 size_t lse_region_bytes(const bd_shape& s, int n_q) {
   size_t bytes = 0;
   for (int n = 1; n <= n_q; ++n) {
+    if (n < n_q && (s.t_ctx + n) % kSKeys != 0) continue;   // the same tiles as the next
     LsePlan lp;
     if (lse_plan(block_context(s, n), n, &lp)) bytes = std::max(bytes, lp.part_bytes);
   }

@@ -396,16 +396,32 @@ static bool tc_streams_better(const bd_shape& s, int n_q) {
   return s.h_q / s.h_kv * n_q <= 21 || units < 128 || units * keys < 5L << 18;
 }
 
-bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
-  const int group = s.h_q / s.h_kv;
-  const long rows_total = (long)group * n_q;
-  const bool ragged = s.seq_lens != nullptr;
-  const bool tc = rows_total > kVMaxRows || (rows_total > kVTcRows && tc_streams_better(s, n_q));
+// What a block's plan depends on beside its row count: the kernel (and its instance), the chunks, the tiles.
+struct VerifyRoute {
+  long rows;            // group * n_q
+  bool tc;              // verify_tc_kernel
+  int nt, chunks, tiles;
+  bool operator==(const VerifyRoute& o) const { return tc == o.tc && nt == o.nt && chunks == o.chunks && tiles == o.tiles; }
+};
+static VerifyRoute verify_route(const bd_shape& s, int n_q) {
+  VerifyRoute r;
+  r.rows = (long)(s.h_q / s.h_kv) * n_q;
+  r.tc = r.rows > kVMaxRows || (r.rows > kVTcRows && tc_streams_better(s, n_q));
   // more query rows than one CTA holds: chunks of equal size
-  const int chunks = tc ? (int)((rows_total + kVTcMaxRows - 1) / kVTcMaxRows) : 1;
+  r.chunks = r.tc ? (int)((r.rows + kVTcMaxRows - 1) / kVTcMaxRows) : 1;
+  r.nt = r.tc ? 0 : r.rows <= 8 ? 1 : 3;
+  const int keys = r.tc ? kVTcKeys : kVKeys;
+  r.tiles = (int)(((long)s.t_ctx + n_q + keys - 1) / keys);
+  return r;
+}
+
+bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
+  const VerifyRoute route = verify_route(s, n_q);
+  const bool ragged = s.seq_lens != nullptr, tc = route.tc;
+  const long rows_total = route.rows;
+  const int chunks = route.chunks, nt = route.nt;
   if (chunks > kVMaxChunks) return false;
   const int nq_rows = (int)((rows_total + chunks - 1) / chunks);
-  const int nt = nq_rows <= 8 ? 1 : 3;
   const int q_tiles = tc ? (nq_rows > 128 ? 2 : 1) : 0;
   KernelInfo k = {nullptr, 0, 0};
   if (!tc) {
@@ -419,8 +435,7 @@ bool verify_plan(const bd_shape& s, int n_q, VerifyPlan* plan) {
   plan->q_tiles = q_tiles;
   plan->nt = nt;
   plan->smem_bytes = tc ? verify_tc_smem(s.head_dim, q_tiles) : k.smem;
-  const long n_keys = (long)s.t_ctx + n_q;
-  plan->tiles_per_unit = (int)((n_keys + keys - 1) / keys);
+  plan->tiles_per_unit = route.tiles;
   const long units = (long)s.batch * s.h_kv * chunks;
   const int tpu = plan->tiles_per_unit;
   const long ctas = std::max(1, current_sm_count() * (tc ? 1 : occupancy(k)));
@@ -472,6 +487,7 @@ size_t verify_partials_bytes(const bd_shape& s, const VerifyPlan& plan) {
 size_t verify_region_bytes(const bd_shape& s, int n_q) {
   size_t bytes = 0;
   for (int n = 1; n <= n_q; ++n) {
+    if (n < n_q && verify_route(s, n) == verify_route(s, n + 1)) continue;   // the longer one needs as much
     VerifyPlan vp;
     if (verify_plan(s, n, &vp)) bytes = std::max(bytes, verify_partials_bytes(s, vp));
   }
